@@ -82,6 +82,133 @@ static std::vector<float> to_f_volume(const std::vector<double>& v, int row, int
   return out;
 }
 
+// Shared-memory layout, packed tables and factor copies of the kernel that runs
+// levels lo .. coarsest in one launch.
+bool MGSolver::build_vsmem(Arena& A, int lo, int n_modes, VSmemArgs& v, std::string& err) {
+  const int nl = int(lv.size());
+  const size_t vb = vbytes();
+  const bool f32c = opt.precision && H.sep_stride > 0;
+  const size_t zf32 = 8 * size_t(lv[nl - 1].nt) * (lv[nl - 1].nr + 1);
+  v.nlev = nl - lo;
+  size_t off = 0;
+  for (int k = 0; k < v.nlev; ++k) {
+    const LevelDev& d = lv[lo + k];
+    v.L[k] = d;
+    v.off_e[k] = int(off);
+    off += size_t(d.nr) * d.nt;
+    v.off_f[k] = int(off);
+    off += size_t(d.nr) * d.nt;
+  }
+  v.tab_off = int(off);
+  // per-slot packed copy of the fused levels' tables and this slot's omega
+  // rows, laid out exactly as the kernel's shared-memory copy: per level,
+  // at the next odd element offset, RT_N x (nr+2) radial and TT_N x (nt+2)
+  // polar entries, then nt r-line and nr polar-line omegas
+  size_t tab = 0;
+  std::vector<size_t> lvl_off(v.nlev);
+  for (int k = 0; k < v.nlev; ++k) {
+    const LevelDev& d = lv[lo + k];
+    tab = (tab + 1) / 2 * 2 + 1;
+    lvl_off[k] = tab;
+    tab += size_t(RT_N) * (d.nr + 2) + size_t(TT_N) * (d.nt + 2) + d.nr + d.nt;
+  }
+  tab = (tab + 3) / 4 * 4;
+  v.tab_stride = int(tab);
+  {
+    const size_t S = size_t(n_modes);
+    std::vector<double> pk(S * tab, 0.0);
+    for (size_t q = 0; q < S; ++q)
+      for (int k = 0; k < v.nlev; ++k) {
+        const LevelHost& h = H.lv[lo + k];
+        const int nr = lv[lo + k].nr, nt = lv[lo + k].nt;
+        double* o = pk.data() + q * tab + lvl_off[k];
+        std::copy(h.rtab.begin(), h.rtab.end(), o);
+        o += size_t(RT_N) * (nr + 2);
+        std::copy(h.ttab.begin(), h.ttab.end(), o);
+        o += size_t(TT_N) * (nt + 2);
+        std::copy(h.om_r.begin() + q * nt, h.om_r.begin() + (q + 1) * nt, o);
+        o += nt;
+        std::copy(h.om_t.begin() + q * nr, h.om_t.begin() + (q + 1) * nr, o);
+      }
+    if (opt.precision) v.tabs = upload(A, to_f(pk));
+    else v.tabs = upload(A, pk);
+    if (!v.tabs) { err = "out of device memory"; return false; }
+  }
+  size_t sbytes = (off * vb + tab * (vb / 2) + 15) / 16 * 16;
+  v.dbl_off = int(sbytes);
+  sbytes += f32c ? zf32 : 32 * size_t(H.nc);
+  v.inv = d_inv;
+  v.blk = d_blk;
+  v.nc = H.nc;
+  v.blk_n = H.blk_n;
+  v.blk_nt = H.blk_nt;
+  v.sep = d_sep;
+  v.sep_stride = H.sep_stride;
+  v.sep_sym = H.sep_sym;
+  const size_t blk_bytes = H.sep_stride > 0
+                               ? size_t(H.sep_stride) * sizeof(double)
+                               : size_t(H.blk_nt) * H.blk_n * (H.blk_n + 2) * sizeof(double);
+  v.blk_smem = ((H.blk_n > 0 || H.sep_stride > 0) && sbytes + blk_bytes <= 220 * 1024) ? 1 : 0;
+  v.blk_off = int(sbytes);
+  v.f32c = f32c ? 1 : 0;
+  v.restage = 0;
+  v.sepf = nullptr;
+  v.sepf_stride = 0;
+  if (f32c) {
+    // the FP32 factor block per slot (see VSmemArgs::sepf), rounded once
+    // from the FP64 factors; staged in its own space when it fits, else
+    // over the first fused level's right-hand side (K >= 2: it is the
+    // kernel's input, staged again from global memory after the coarsest
+    // solve), else read from global memory
+    const int nrc = lv[nl - 1].nr, ntc = lv[nl - 1].nt, vr = H.sep_sym ? ntc / 2 : ntc;
+    const size_t ncc = size_t(nrc) * ntc;
+    const size_t pc = size_t(ntc) * (nrc + 1);   // padded rows
+    v.sepf_stride = int((2 * size_t(vr) * ntc + 3 * pc + 3) / 4 * 4);
+    if (!d_sepf) {
+      const size_t S_ = size_t(n_modes);
+      std::vector<float> pf(S_ * size_t(v.sepf_stride), 0.f);
+      for (size_t q = 0; q < S_; ++q) {
+        const double* Vm = H.coarse_sep.data() + q * H.sep_stride;   // [vr][nt]
+        const double* Vi = Vm + size_t(vr) * ntc;                     // [nt][vr]
+        const double* rest = Vi + size_t(ntc) * vr;                   // 1/pivot, upper, lower
+        float* o = pf.data() + q * v.sepf_stride;
+        for (int j = 0; j < vr; ++j)
+          for (int k = 0; k < ntc; ++k) o[size_t(j) * ntc + k] = float(Vi[size_t(k) * vr + j]);
+        o += size_t(vr) * ntc;
+        for (int k = 0; k < ntc; ++k)
+          for (int j = 0; j < vr; ++j) o[size_t(k) * vr + j] = float(Vm[size_t(j) * ntc + k]);
+        o += size_t(ntc) * vr;
+        for (int t = 0; t < 3; ++t)
+          for (int k = 0; k < ntc; ++k)
+            for (int i = 0; i < nrc; ++i) o[t * pc + size_t(k) * (nrc + 1) + i] = float(rest[t * ncc + size_t(k) * nrc + i]);
+      }
+      d_sepf = upload(A, pf);
+    }
+    v.sepf = d_sepf;
+    if (!v.sepf) { err = "out of device memory"; return false; }
+    const size_t fac = 4 * size_t(v.sepf_stride);
+    const size_t f0 = size_t(v.L[0].nr) * v.L[0].nt * vb;
+    if (sbytes + fac <= 224 * 1024) {
+      v.blk_smem = 1;
+    } else if (v.nlev >= 2 && fac <= f0) {
+      v.blk_smem = 1;
+      v.restage = 1;
+      v.blk_off = int(size_t(v.off_f[0]) * vb);
+    } else {
+      v.blk_smem = 0;
+    }
+    if (v.blk_smem && !v.restage) sbytes += fac;
+  } else if (v.blk_smem) {
+    sbytes += blk_bytes;
+  }
+  v.smem_bytes = sbytes + 16;
+  if (H.nc < 16 || (H.nc & (H.nc - 1))) { err = "coarsest level must have a power-of-two size >= 16"; return false; }
+  v.nu1 = opt.nu1;
+  v.nu2 = opt.nu2;
+  v.n_sor = opt.n_sor;
+  return true;
+}
+
 bool MGSolver::init(Arena& A, const PlaneGeo& fine, bool neumann, const std::vector<int>& modes,
                     const std::vector<int>& plane_slot, int mp, const MGOptions& o,
                     std::string& err) {
@@ -182,120 +309,21 @@ bool MGSolver::init(Arena& A, const PlaneGeo& fine, bool neumann, const std::vec
       if (bytes > budget || lv[l].nr > 128 || lv[l].nt > 128 || nl - l > 8) break;
       first = l;
     }
-    vs.nlev = nl - first;
-    size_t off = 0;
-    for (int k = 0; k < vs.nlev; ++k) {
-      const LevelDev& d = lv[first + k];
-      vs.L[k] = d;
-      vs.off_e[k] = int(off);
-      off += size_t(d.nr) * d.nt;
-      vs.off_f[k] = int(off);
-      off += size_t(d.nr) * d.nt;
-    }
-    vs.tab_off = int(off);
-    // per-slot packed copy of the fused levels' tables and this slot's omega
-    // rows, laid out exactly as the kernel's shared-memory copy: per level,
-    // at the next odd element offset, RT_N x (nr+2) radial and TT_N x (nt+2)
-    // polar entries, then nt r-line and nr polar-line omegas
-    size_t tab = 0;
-    std::vector<size_t> lvl_off(vs.nlev);
-    for (int k = 0; k < vs.nlev; ++k) {
-      const LevelDev& d = lv[first + k];
-      tab = (tab + 1) / 2 * 2 + 1;
-      lvl_off[k] = tab;
-      tab += size_t(RT_N) * (d.nr + 2) + size_t(TT_N) * (d.nt + 2) + d.nr + d.nt;
-    }
-    tab = (tab + 3) / 4 * 4;
-    vs.tab_stride = int(tab);
-    {
-      const size_t S = modes.size();
-      std::vector<double> pk(S * tab, 0.0);
-      for (size_t q = 0; q < S; ++q)
-        for (int k = 0; k < vs.nlev; ++k) {
-          const LevelHost& h = H.lv[first + k];
-          const int nr = lv[first + k].nr, nt = lv[first + k].nt;
-          double* o = pk.data() + q * tab + lvl_off[k];
-          std::copy(h.rtab.begin(), h.rtab.end(), o);
-          o += size_t(RT_N) * (nr + 2);
-          std::copy(h.ttab.begin(), h.ttab.end(), o);
-          o += size_t(TT_N) * (nt + 2);
-          std::copy(h.om_r.begin() + q * nt, h.om_r.begin() + (q + 1) * nt, o);
-          o += nt;
-          std::copy(h.om_t.begin() + q * nr, h.om_t.begin() + (q + 1) * nr, o);
-        }
-      if (opt.precision) vs.tabs = upload(A, to_f(pk));
-      else vs.tabs = upload(A, pk);
-      if (!vs.tabs) { err = "out of device memory"; return false; }
-    }
-    size_t sbytes = (off * vb + tab * (vb / 2) + 15) / 16 * 16;
-    vs.dbl_off = int(sbytes);
-    sbytes += f32c ? zf32 : 32 * size_t(H.nc);
-    vs.inv = d_inv;
-    vs.blk = d_blk;
-    vs.nc = H.nc;
-    vs.blk_n = H.blk_n;
-    vs.blk_nt = H.blk_nt;
-    vs.sep = d_sep;
-    vs.sep_stride = H.sep_stride;
-    vs.sep_sym = H.sep_sym;
-    const size_t blk_bytes = H.sep_stride > 0
-                                 ? size_t(H.sep_stride) * sizeof(double)
-                                 : size_t(H.blk_nt) * H.blk_n * (H.blk_n + 2) * sizeof(double);
-    vs.blk_smem = ((H.blk_n > 0 || H.sep_stride > 0) && sbytes + blk_bytes <= 220 * 1024) ? 1 : 0;
-    vs.blk_off = int(sbytes);
-    vs.f32c = f32c ? 1 : 0;
-    vs.restage = 0;
-    vs.sepf = nullptr;
-    vs.sepf_stride = 0;
-    if (f32c) {
-      // the FP32 factor block per slot (see VSmemArgs::sepf), rounded once
-      // from the FP64 factors; staged in its own space when it fits, else
-      // over the first fused level's right-hand side (K >= 2: it is the
-      // kernel's input, staged again from global memory after the coarsest
-      // solve), else read from global memory
-      const int nrc = lv[nl - 1].nr, ntc = lv[nl - 1].nt, vr = H.sep_sym ? ntc / 2 : ntc;
-      const size_t ncc = size_t(nrc) * ntc;
-      const size_t pc = size_t(ntc) * (nrc + 1);   // padded rows
-      vs.sepf_stride = int((2 * size_t(vr) * ntc + 3 * pc + 3) / 4 * 4);
-      const size_t S_ = modes.size();
-      std::vector<float> pf(S_ * size_t(vs.sepf_stride), 0.f);
-      for (size_t q = 0; q < S_; ++q) {
-        const double* Vm = H.coarse_sep.data() + q * H.sep_stride;   // [vr][nt]
-        const double* Vi = Vm + size_t(vr) * ntc;                     // [nt][vr]
-        const double* rest = Vi + size_t(ntc) * vr;                   // 1/pivot, upper, lower
-        float* o = pf.data() + q * vs.sepf_stride;
-        for (int j = 0; j < vr; ++j)
-          for (int k = 0; k < ntc; ++k) o[size_t(j) * ntc + k] = float(Vi[size_t(k) * vr + j]);
-        o += size_t(vr) * ntc;
-        for (int k = 0; k < ntc; ++k)
-          for (int j = 0; j < vr; ++j) o[size_t(k) * vr + j] = float(Vm[size_t(j) * ntc + k]);
-        o += size_t(ntc) * vr;
-        for (int t = 0; t < 3; ++t)
-          for (int k = 0; k < ntc; ++k)
-            for (int i = 0; i < nrc; ++i) o[t * pc + size_t(k) * (nrc + 1) + i] = float(rest[t * ncc + size_t(k) * nrc + i]);
-      }
-      vs.sepf = upload(A, pf);
-      if (!vs.sepf) { err = "out of device memory"; return false; }
-      const size_t fac = 4 * size_t(vs.sepf_stride);
-      const size_t f0 = size_t(vs.L[0].nr) * vs.L[0].nt * vb;
-      if (sbytes + fac <= 224 * 1024) {
-        vs.blk_smem = 1;
-      } else if (vs.nlev >= 2 && fac <= f0) {
-        vs.blk_smem = 1;
-        vs.restage = 1;
-        vs.blk_off = int(size_t(vs.off_f[0]) * vb);
-      } else {
-        vs.blk_smem = 0;
-      }
-      if (vs.blk_smem && !vs.restage) sbytes += fac;
-    } else if (vs.blk_smem) {
-      sbytes += blk_bytes;
-    }
-    vs.smem_bytes = sbytes + 16;
-    if (H.nc < 16 || (H.nc & (H.nc - 1))) { err = "coarsest level must have a power-of-two size >= 16"; return false; }
-    vs.nu1 = opt.nu1;
-    vs.nu2 = opt.nu2;
-    vs.n_sor = opt.n_sor;
+  }
+  if (!build_vsmem(A, first, int(modes.size()), vs, err)) return false;
+  base = first;
+  vsb = vs;
+  if (!opt.precision && nl - 1 > first) {
+    // FP64 path: a solve's V-cycle smooths every level with the level-wide
+    // line passes and leaves one block per plane only the coarsest solve.  A
+    // line relaxation is FP64 arithmetic throughout and one SM's FP64 pipe
+    // does 2 operations a clock, so a plane's 64 x 32 level cost one block 190
+    // of its 203 us whatever the number of planes; spread over the SMs the
+    // level's eight passes and transfers take 68 us with one plane active
+    // and 11.2 -> 7.9 ms a solve (128 x 64 x 128, tol 1e-10).  The mixed path
+    // keeps the levels together: its passes are short of FP32 work, not SMs.
+    base = nl - 1;
+    if (!build_vsmem(A, base, int(modes.size()), vsb, err)) return false;
   }
   const int nblk = residual_blocks(lv[0].nr, lv[0].nt);
   d_act = static_cast<int*>(A.get(sizeof(int) * mp));
@@ -417,11 +445,11 @@ void MGSolver::prolong(int l, void* ee, const void* ec, cudaStream_t st) {
   else
     launch_prolong<double>(lv[l], lv[l + 1], batch, (double2*)ee, (const double2*)ec, st);
 }
-void MGSolver::fused(cudaStream_t st) {
+void MGSolver::fused(int lo, const VSmemArgs& v, cudaStream_t st) {
   if (opt.precision)
-    launch_vsmem<float>(vs, batch, (const float2*)f[first], (float2*)e[first], st);
+    launch_vsmem<float>(v, batch, (const float2*)f[lo], (float2*)e[lo], st);
   else
-    launch_vsmem<double>(vs, batch, (const double2*)f[first], (double2*)e[first], st);
+    launch_vsmem<double>(v, batch, (const double2*)f[lo], (double2*)e[lo], st);
 }
 void MGSolver::residual(const double2* ff, const double2* u, double tol, cudaStream_t st,
                         int use_cond, unsigned long long cond) {
@@ -461,22 +489,24 @@ void MGSolver::residual_to(const double2* ff, const double2* u, void* r, cudaStr
 // One V-cycle on the error equation L e_0 = f_0 (f_0 = FP64 residual in the
 // buffer precision), e_0 starting from zero (Sec. 3: pre-smoothing, defect
 // restriction, coarse correction, prolongation, post-smoothing).  Levels
-// below `first` run as level-wide kernels over all active planes; the rest
+// below `base` run as level-wide kernels over all active planes; the rest
 // runs in the shared-memory kernel, one block per plane.
 // With post-smoothing on level 0, the update (with u) rides on its last pass.
 bool MGSolver::vcycle(cudaStream_t st, double2* u) {
-  for (int l = 0; l < first; ++l) {
-    if (opt.nu1 > 0) smooth(l, e[l], f[l], opt.nu1, true, st);
+  for (int l = 0; l < base; ++l) {
+    const int nu1 = l >= first ? vs.nu1 : opt.nu1;
+    if (nu1 > 0) smooth(l, e[l], f[l], nu1, true, st);
     else cudaMemsetAsync(e[l], 0, size_t(max_planes) * lv[l].nr * lv[l].nt * vbytes(), st);
     restrict_(l, e[l], f[l], f[l + 1], st);
   }
-  fused(st);
+  fused(base, vsb, st);
   bool updated = false;
-  for (int l = first - 1; l >= 0; --l) {
+  for (int l = base - 1; l >= 0; --l) {
     prolong(l, e[l], e[l + 1], st);
-    if (opt.nu2 > 0) {
+    const int nu2 = l >= first ? vs.nu2 : opt.nu2;
+    if (nu2 > 0) {
       double2* uu = l == 0 ? u : nullptr;
-      smooth(l, e[l], f[l], opt.nu2, false, st, uu);
+      smooth(l, e[l], f[l], nu2, false, st, uu);
       updated = uu != nullptr;
     }
   }
@@ -488,9 +518,9 @@ void MGSolver::set_schedule(int nu1, int nu2, int n_sor, Tiles tiles, int nu1f, 
   opt.nu2 = nu2;
   opt.nu1f = nu1f;
   opt.nu2f = nu2f;
-  vs.nu1 = nu1f > 0 ? nu1f : nu1;
-  vs.nu2 = nu2f > 0 ? nu2f : nu2;
-  opt.n_sor = vs.n_sor = n_sor;
+  vs.nu1 = vsb.nu1 = nu1f > 0 ? nu1f : nu1;
+  vs.nu2 = vsb.nu2 = nu2f > 0 ? nu2f : nu2;
+  opt.n_sor = vs.n_sor = vsb.n_sor = n_sor;
   opt.tiles = tiles;
   prepare_tail();
 }

@@ -78,7 +78,10 @@ class MGSolver {
   // level buffers (T2 of the precision): e[l], f[l]
   std::vector<void*> e, f;
   void* tmp = nullptr;             // ping-pong buffer of the global-memory smoother
-  int first = 0;                   // first level handled by the shared-memory kernel
+  int first = 0;                   // first level the shared-memory kernel can take
+  // the level from which a solve's V-cycle runs it, and its arguments there
+  int base = 0;
+  VSmemArgs vsb{};
   int zero_guess = 0;              // the next solve starts from u = 0 (set by the caller)
   VSmemArgs vs{};
   // stage helpers on explicit buffers
@@ -87,7 +90,9 @@ class MGSolver {
               double2* u = nullptr);
   void restrict_(int level, const void* e, const void* f, void* fc, cudaStream_t st);
   void prolong(int level, void* e, const void* ec, cudaStream_t st);
-  void fused(cudaStream_t st);   // levels first .. coarsest in shared memory
+  // levels lo .. coarsest in shared memory, with v built for lo
+  void fused(int lo, const VSmemArgs& v, cudaStream_t st);
+  bool build_vsmem(Arena& A, int lo, int n_modes, VSmemArgs& v, std::string& err);
   void residual(const double2* f, const double2* u, double tol, cudaStream_t st, int use_cond,
                 unsigned long long cond);
   // the defect alone into r (tolerance 0: no plane retires)
@@ -101,6 +106,7 @@ class MGSolver {
   double* d_inv = nullptr;
   double* d_blk = nullptr;
   double* d_sep = nullptr;
+  float* d_sepf = nullptr;
   double* d_ctab = nullptr;   // level-0 per-cell FP64 products [4][nt][nr]
   double* d_dtab = nullptr;   // level-0 diagonal of each mode slot [slots][nt][nr]
   SqPart* d_part = nullptr;
