@@ -40,7 +40,7 @@ struct psolve_ctx {
   std::vector<BPoint> bp;
   BDev bdev{};
   double* gt = nullptr;
-  double2* tw = nullptr;
+  FftTables fft;
   double2 *u = nullptr, *f = nullptr, *sigma = nullptr, *theta = nullptr;
   // warm start: the previous solve's Psi and Phi mode planes as initial guesses
   double2 *psi_prev = nullptr, *phi_prev = nullptr;
@@ -227,11 +227,10 @@ static int create_impl(psolve_t* out, const psolve_desc* din, int nd) {
   }
   h->u = static_cast<double2*>(h->A.get(sizeof(double2) * plane * P));
   h->f = static_cast<double2*>(h->A.get(sizeof(double2) * plane * P));
-  // twiddles e^{-2 pi i k / N}
-  std::vector<double2> tw(d.n_phi / 2);
-  for (int k = 0; k < d.n_phi / 2; ++k)
-    tw[k] = make_double2(std::cos(2.0 * kPi * k / d.n_phi), -std::sin(2.0 * kPi * k / d.n_phi));
-  h->tw = static_cast<double2*>(h->A.get(sizeof(double2) * tw.size()));
+  // twiddles of the transforms; the forward one scales by 4 pi G / N
+  size_t inv_at = 0;
+  const std::vector<int4> tw = fft_tables(d.n_phi, 4.0 * kPi * d.G / d.n_phi, &h->fft, &inv_at);
+  int4* d_tw = static_cast<int4*>(h->A.get(sizeof(int4) * tw.size()));
   // boundary points, screening and coupling coefficients
   h->bp = boundary_points(h->g);
   h->nb = int(h->bp.size());
@@ -283,11 +282,13 @@ static int create_impl(psolve_t* out, const psolve_desc* din, int nd) {
     s->iter = static_cast<int*>(h->A.get(sizeof(int)));
   }
   h->d_worst = static_cast<int*>(h->A.get(sizeof(int)));
-  if (!h->u || !h->f || !h->tw || !h->gt || !h->theta || !h->d_worst || !h->sf.iter) {
+  if (!h->u || !h->f || !d_tw || !h->gt || !h->theta || !h->d_worst || !h->sf.iter) {
     h->A.release_all();
     return fail(PSOLVE_ERR_NOMEM, "out of device memory");
   }
-  cudaMemcpy(h->tw, tw.data(), sizeof(double2) * tw.size(), cudaMemcpyHostToDevice);
+  cudaMemcpy(d_tw, tw.data(), sizeof(int4) * tw.size(), cudaMemcpyHostToDevice);
+  h->fft.fwd = d_tw;
+  h->fft.inv = d_tw + inv_at;
   cudaMallocHost(&h->h_worst, sizeof(int));
   for (cudaEvent_t& e : h->mark)
     if (cudaEventCreate(&e) != cudaSuccess) e = nullptr;
@@ -511,7 +512,7 @@ static void enqueue_front(psolve_t h, const double* rho) {
   mark(h, 0);
   for (int b = 0; b < h->nd; ++b)
     launch_fft_forward(rho + b * cells(h), h->f + size_t(b) * h->M * mode_plane(h), h->d.n_r, h->d.n_tz,
-                       h->d.n_phi, 4.0 * kPi * h->d.G / h->d.n_phi, h->tw, h->st);
+                       h->d.n_phi, h->fft, h->st);
   mark(h, 1);
   if (warm_state(h) == 2)
     cudaMemcpyAsync(h->u, h->psi_prev, plane_bytes(h), cudaMemcpyDeviceToDevice, h->st);
@@ -543,7 +544,7 @@ static void enqueue_back(psolve_t h, double* phi) {
   if (h->warm) cudaMemcpyAsync(h->phi_prev, h->u, plane_bytes(h), cudaMemcpyDeviceToDevice, h->st);
   for (int b = 0; b < h->nd; ++b)
     launch_fft_inverse(h->u + size_t(b) * h->M * mode_plane(h), phi + b * cells(h), h->d.n_r, h->d.n_tz,
-                       h->d.n_phi, h->tw, h->st);
+                       h->d.n_phi, h->fft, h->st);
   k_worst<<<1, 256, 0, h->st>>>(h->sp.status, h->sf.status, h->P, h->d_worst);
   cudaMemcpyAsync(h->h_worst, h->d_worst, sizeof(int), cudaMemcpyDeviceToHost, h->st);
   mark(h, 5);
@@ -1191,7 +1192,7 @@ extern "C" int psolve_get_stats(psolve_t h, psolve_stats* s) {
 extern "C" int psolve_stage_forward(psolve_t h, const double* rho, double* f_hat) {
   if (!h || !rho || !f_hat) return fail(PSOLVE_ERR_ARG, "null argument");
   launch_fft_forward(rho, reinterpret_cast<double2*>(f_hat), h->d.n_r, h->d.n_tz, h->d.n_phi,
-                     4.0 * kPi * h->d.G / h->d.n_phi, h->tw, h->st);
+                     h->fft, h->st);
   return cudaStreamSynchronize(h->st) == cudaSuccess && cuda_ok("forward") ? PSOLVE_OK
                                                                              : PSOLVE_ERR_CUDA;
 }
@@ -1201,7 +1202,7 @@ extern "C" int psolve_stage_forward_rows(psolve_t h, const double* rho_rows, int
   if (!h || !rho_rows || !f_hat_rows) return fail(PSOLVE_ERR_ARG, "null argument");
   if (n_rows < 1 || n_rows > h->d.n_r) return fail(PSOLVE_ERR_ARG, "n_rows must lie in 1..n_r");
   launch_fft_forward(rho_rows, reinterpret_cast<double2*>(f_hat_rows), n_rows, h->d.n_tz, h->d.n_phi,
-                     4.0 * kPi * h->d.G / h->d.n_phi, h->tw, h->st);
+                     h->fft, h->st);
   return cudaStreamSynchronize(h->st) == cudaSuccess && cuda_ok("forward_rows") ? PSOLVE_OK
                                                                                   : PSOLVE_ERR_CUDA;
 }
@@ -1211,7 +1212,7 @@ extern "C" int psolve_stage_inverse_rows(psolve_t h, const double* phi_hat_rows,
   if (!h || !phi_hat_rows || !phi_rows) return fail(PSOLVE_ERR_ARG, "null argument");
   if (n_rows < 1 || n_rows > h->d.n_r) return fail(PSOLVE_ERR_ARG, "n_rows must lie in 1..n_r");
   launch_fft_inverse(reinterpret_cast<const double2*>(phi_hat_rows), phi_rows, n_rows, h->d.n_tz,
-                     h->d.n_phi, h->tw, h->st);
+                     h->d.n_phi, h->fft, h->st);
   return cudaStreamSynchronize(h->st) == cudaSuccess && cuda_ok("inverse_rows") ? PSOLVE_OK
                                                                                   : PSOLVE_ERR_CUDA;
 }
@@ -1261,7 +1262,7 @@ extern "C" int psolve_solve_modes(psolve_t h, const int* modes_host, int n, cons
 extern "C" int psolve_stage_inverse(psolve_t h, const double* phi_hat, double* phi) {
   if (!h || !phi_hat || !phi) return fail(PSOLVE_ERR_ARG, "null argument");
   launch_fft_inverse(reinterpret_cast<const double2*>(phi_hat), phi, h->d.n_r, h->d.n_tz,
-                     h->d.n_phi, h->tw, h->st);
+                     h->d.n_phi, h->fft, h->st);
   return cudaStreamSynchronize(h->st) == cudaSuccess && cuda_ok("inverse") ? PSOLVE_OK
                                                                              : PSOLVE_ERR_CUDA;
 }

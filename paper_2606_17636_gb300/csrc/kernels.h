@@ -192,11 +192,22 @@ struct Batch {
 };
 
 // ---- FFT (k_fft.cu) --------------------------------------------------------
+// Twiddle tables of a handle's transforms in device memory (fft_tables).  The
+// forward ones carry the scale's mantissa and es its power of two; lengths up
+// to 16 have no twiddles and multiply their outputs by post.
+struct FftTables {
+  const int4* fwd = nullptr;
+  const int4* inv = nullptr;
+  int es = 0;
+  double post = 1.0;
+  int bad = 0;   // the scale is not finite
+};
+std::vector<int4> fft_tables(int N, double scale, FftTables* t, size_t* inv_at);
 // f[m][j][i] (double2) = scale * sum_k rho[i][j][k] e^{-2 pi i m k / N}
-void launch_fft_forward(const double* rho, double2* f, int nr, int nt, int N, double scale,
-                        const double2* tw, cudaStream_t st);
-void launch_fft_inverse(const double2* fh, double* phi, int nr, int nt, int N,
-                        const double2* tw, cudaStream_t st);
+void launch_fft_forward(const double* rho, double2* f, int nr, int nt, int N, const FftTables& tab,
+                        cudaStream_t st);
+void launch_fft_inverse(const double2* fh, double* phi, int nr, int nt, int N, const FftTables& tab,
+                        cudaStream_t st);
 
 // ---- multigrid (k_mg.cu), T = float or double ---------------------------------
 // Tile shapes of the level-wide smoothing passes: radial lines per block
