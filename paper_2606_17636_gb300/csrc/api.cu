@@ -550,10 +550,18 @@ static void enqueue_back(psolve_t h, double* phi) {
   mark(h, 5);
 }
 
-static int add_while(psolve_t h, cudaGraph_t graph, double tol, cudaStream_t body_st) {
+// The second phase of a multigrid loop runs when the first one handed planes
+// over (continue flag 2).
+__global__ void k_hand_over(const int* cont, cudaGraphConditionalHandle cond) {
+  cudaGraphSetConditional(cond, *cont == 2 ? 1u : 0u);
+}
+
+static int add_while(psolve_t h, cudaGraph_t graph, double tol, cudaStream_t body_st, bool few) {
   cudaGraphConditionalHandle cond;
-  if (cudaGraphConditionalHandleCreate(&cond, graph, 1, cudaGraphCondAssignDefault) != cudaSuccess)
+  const bool second = few && h->mg.many_phase();
+  if (cudaGraphConditionalHandleCreate(&cond, graph, second ? 0 : 1, cudaGraphCondAssignDefault) != cudaSuccess)
     return -1;
+  if (second) k_hand_over<<<1, 1, 0, h->st>>>(h->mg.d_cont, cond);
   cudaStreamCaptureStatus cs;
   const cudaGraphNode_t* deps = nullptr;
   size_t ndeps = 0;
@@ -574,10 +582,17 @@ static int add_while(psolve_t h, cudaGraph_t graph, double tol, cudaStream_t bod
   if (cudaStreamBeginCaptureToGraph(body_st, body, nullptr, nullptr, 0,
                                     cudaStreamCaptureModeRelaxed) != cudaSuccess)
     return -1;
-  h->mg.loop_body(h->f, h->u, tol, body_st, 1, cond);
+  h->mg.loop_body(h->f, h->u, tol, body_st, 1, cond, few);
   cudaGraph_t out;
-  if (cudaStreamEndCapture(body_st, &out) != cudaSuccess) return -1;
-  h->mg.tail(h->f, h->u, tol, h->st);   // planes the loop handed over (none: returns at once)
+  return cudaStreamEndCapture(body_st, &out) == cudaSuccess ? 0 : -1;
+}
+
+// A multigrid solve: its loops and the tail kernel, each taking the planes that
+// the one before handed over (none: it returns at once).
+static int add_loops(psolve_t h, cudaGraph_t graph, double tol, cudaStream_t body_st) {
+  if (h->mg.many_phase() && add_while(h, graph, tol, body_st, false)) return -1;
+  if (h->mg.few_phase() && add_while(h, graph, tol, body_st, true)) return -1;
+  h->mg.tail(h->f, h->u, tol, h->st);
   return 0;
 }
 
@@ -600,10 +615,10 @@ static int capture(psolve_t h, const double* rho, double* phi, double tol) {
     rc = -1;
   if (!rc) {
     enqueue_front(h, rho);
-    rc = add_while(h, graph, tol, body_st);
+    rc = add_loops(h, graph, tol, body_st);
     if (!rc) {
       enqueue_middle(h);
-      rc = add_while(h, graph, tol, body_st);
+      rc = add_loops(h, graph, tol, body_st);
     }
     if (!rc) enqueue_back(h, phi);
     cudaGraph_t g2;
@@ -853,10 +868,10 @@ extern "C" int psolve_batch_create(psolve_batch_t* out, psolve_t* hs, const doub
       h->st = b->branch[k];
       cudaStreamWaitEvent(h->st, fork, 0);
       enqueue_front(h, rhos[k]);
-      rc = add_while(h, graph, tol, body);
+      rc = add_loops(h, graph, tol, body);
       if (!rc) {
         enqueue_middle(h);
-        rc = add_while(h, graph, tol, body);
+        rc = add_loops(h, graph, tol, body);
       }
       if (!rc) {
         enqueue_back(h, phis[k]);

@@ -5,7 +5,9 @@
 // overwritten by another block.  The first colour-1 neighbour that belongs to
 // the next block is recomputed from e_in (one extra line or column per block),
 // giving exactly the values the two-launch ordering produces.  A smoothing
-// cycle is a radial pass e -> tmp followed by a polar pass tmp -> e.
+// cycle is a radial pass e -> tmp followed by a polar pass tmp -> e.  FP32 levels
+// of enough cells take the passes of k_band.cu instead (band_pays there has the
+// rule and both sides' times); FP64 levels and the others stay here.
 //
 // Tile shapes: a radial block owns Wmax = 8 or 4 lines (one warp per line),
 // a polar block TWmax columns (8, 16 or 32; at most 160 KB of staged tile);
@@ -301,9 +303,20 @@ void launch_smooth(const LevelDev& L, const Batch& B, vec2_t<T>* e, const vec2_t
                    vec2_t<T>* tmp, int cycles, int n_sor, bool zero_init, Tiles tiles,
                    cudaStream_t st, double2* u) {
   const int Wmax = rpass_lines(L.nr, sizeof(vec2_t<T>), tiles.lines_r == 4 ? 4 : 8);
+  bool band = false;   // passes of k_band.cu
+  if constexpr (sizeof(T) == 4) band = band_pays(L.nr, L.nt, n_sor, B.max_planes);
   for (int c = 0; c < cycles; ++c) {
-    rpass2_any<T>(L, B, e, tmp, f, zero_init && c == 0, n_sor, Wmax, st);
-    tpass2_any<T>(L, B, tmp, e, f, n_sor, tiles.cols_t, c == cycles - 1 ? u : nullptr, st);
+    const bool zi = zero_init && c == 0;
+    double2* uu = c == cycles - 1 ? u : nullptr;
+    if (band) {
+      if constexpr (sizeof(T) == 4) {
+        launch_band_radial(L, B, e, tmp, f, zi, n_sor, st);
+        launch_march(L, B, tmp, e, f, n_sor, uu, st);
+      }
+    } else {
+      rpass2_any<T>(L, B, e, tmp, f, zi, n_sor, Wmax, st);
+      tpass2_any<T>(L, B, tmp, e, f, n_sor, tiles.cols_t, uu, st);
+    }
   }
 }
 

@@ -74,6 +74,18 @@ __device__ __forceinline__ double f32_to_f64(float x) {
   }
   return __longlong_as_double(static_cast<long long>(d));
 }
+// The same for streams of values (the refinement's update): the cases beyond
+// normal values and zero behind a call, so that the common ones take six
+// instructions instead of the 20 and more of all cases as selects.  Update
+// fused into the polar march, 129 planes of 256 x 128: 66 -> 61 us, one
+// plane 10.0 -> 8.7.  (Kernels that are short of registers keep the form above.)
+static __device__ __noinline__ double f32_to_f64_rare(float x) { return f32_to_f64(x); }
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x), a = b & 0x7fffffffu;
+  if (a - 0x800000u >= 0x7f000000u && a != 0u) return f32_to_f64_rare(x);
+  const unsigned hi = a ? (a >> 3) + 0x38000000u : 0u;
+  return __hiloint2double(int(hi | (b & 0x80000000u)), int(b << 29));
+}
 
 // Volume-weighted sums of squares in FP32 over the whole binary64 range.  A
 // sum is an FP32 value s with an exponent e and stands for s 2^(2e): every
@@ -155,7 +167,7 @@ __device__ __forceinline__ T to_buf(double x) {
 }
 template <typename T>
 __device__ __forceinline__ double from_buf(T x) {
-  if constexpr (sizeof(T) == sizeof(float)) return f32_to_f64(x);
+  if constexpr (sizeof(T) == sizeof(float)) return widen(x);
   else return x;
 }
 #endif
@@ -232,6 +244,36 @@ template <typename T>
 void launch_smooth(const LevelDev& L, const Batch& B, vec2_t<T>* e, const vec2_t<T>* f,
                    vec2_t<T>* tmp, int cycles, int n_sor, bool zero_init, Tiles tiles,
                    cudaStream_t st, double2* u = nullptr);
+
+// The same passes for FP32 lines of 32 to 512 cells held in registers
+// (k_band.cu: radial bands, polar marches), where they pay.
+bool band_pays(int nr, int nt, int n_sor, int planes);
+void launch_band_radial(const LevelDev& L, const Batch& B, const float2* ein, float2* eout, const float2* f,
+                        bool zero_init, int n_sor, cudaStream_t st);
+void launch_march(const LevelDev& L, const Batch& B, const float2* ein, float2* eout, const float2* f, int n_sor,
+                  double2* u, cudaStream_t st);
+
+// Several smoothing passes of a level per launch on overlapping windows
+// (k_tile.cu, FP32).
+enum { TILE_PROLONG = 1, TILE_RESTRICT = 2, TILE_UPDATE = 4 };
+struct TileStep {
+  int npass;             // passes, radial first
+  int halo, ntx, nty;    // halo cells of the windows and their counts along r and theta / z
+  int op;                // TILE_* steps before and after the passes
+  int n_sor;
+  const float2* src;     // the error's planes before the passes (nullptr: zero)
+  float2* dst;           // and after them (not written with TILE_UPDATE); never src
+  const float2* f;       // right-hand side
+  const float2* ec;      // TILE_PROLONG: the next coarser level's error
+  float2* fc;            // TILE_RESTRICT: the next coarser level's right-hand side
+  double2* u;            // TILE_UPDATE: FP64 solution that the result is added to
+};
+// Fills t's passes, halo and window counts for `cycles` smoothing cycles;
+// false when a line is shorter than a window or the halo leaves a window less
+// than 16 cells of its own.
+bool tile_step(int nr, int nt, int n_sor, int cycles, bool restricts, TileStep& t);
+int tile_slots(int nr, int nt);   // windows resident at once
+void launch_tile(const LevelDev& L, const LevelDev& C, const Batch& B, const TileStep& a, cudaStream_t st);
 
 // Lower part of a V-cycle in shared memory, one block per plane (k_vsmem.cu).
 struct VSmemArgs {

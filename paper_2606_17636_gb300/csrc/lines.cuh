@@ -382,4 +382,41 @@ __device__ __forceinline__ void relax_t(const LevelDev& L, const T* rt, const T*
   sor_line<T, CPL>(ev, g, up, dn, id, w, nt, n_sor);
 }
 
+// ---- runs of consecutive cells per lane (FP32) ----------------------------------
+// Packed multiply-adds on the two components of a cell with one coefficient.
+__device__ __forceinline__ float2 fma2(float a, float2 b, float2 c) { return __ffma2_rn(make_float2(a, a), b, c); }
+__device__ __forceinline__ float2 mul2(float a, float2 b) { return __fmul2_rn(make_float2(a, a), b); }
+
+// n_sor even-odd sweeps of a line of which the lane holds CPL consecutive cells
+// (the first one even) and lanes SH apart the next; zero beyond the first and
+// last lane.  The operations of every cell are sor_line's, with the
+// signs moved into the coefficients (nup = -up, ndn = -dn, nid = -id, nw = -w;
+// exact), so the results are bitwise the same; a half-sweep takes one shuffle
+// per component instead of one per pair of cells.
+template <int CPL, int SH = 1>
+__device__ __forceinline__ void sor_run(float2 (&e)[CPL], const float2 (&g)[CPL], const float (&nup)[CPL],
+                                        const float (&ndn)[CPL], const float (&nid)[CPL], float nw, bool first,
+                                        bool last, int n_sor) {
+  auto upd = [&](int c, float2 em, float2 ep) {
+    const float2 r = fma2(ndn[c], em, fma2(nup[c], ep, g[c]));
+    e[c] = fma2(nw, fma2(nid[c], r, e[c]), e[c]);
+  };
+#pragma unroll 1
+  for (int it = 0; it < n_sor; ++it) {
+    float2 l, r;
+    l.x = __shfl_up_sync(0xffffffffu, e[CPL - 1].x, SH);
+    l.y = __shfl_up_sync(0xffffffffu, e[CPL - 1].y, SH);
+    if (first) l = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int c = 2; c < CPL; c += 2) upd(c, e[c - 1], e[c + 1]);
+    upd(0, l, e[1]);
+    r.x = __shfl_down_sync(0xffffffffu, e[0].x, SH);
+    r.y = __shfl_down_sync(0xffffffffu, e[0].y, SH);
+    if (last) r = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int c = 1; c < CPL - 1; c += 2) upd(c, e[c - 1], e[c + 1]);
+    upd(CPL - 1, e[CPL - 2], r);
+  }
+}
+
 }  // namespace ps

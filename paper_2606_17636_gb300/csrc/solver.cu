@@ -325,6 +325,16 @@ bool MGSolver::init(Arena& A, const PlaneGeo& fine, bool neumann, const std::vec
     base = nl - 1;
     if (!build_vsmem(A, base, int(modes.size()), vsb, err)) return false;
   }
+  if (opt.precision && base > 0) {   // the window passes' buffers; without them every plane stays with the level-wide passes
+    tmp2 = A.get(size_t(mp) * lv[0].nr * lv[0].nt * vb);
+    e2.assign(nl, nullptr);
+    for (int l = 1; l < base && tmp2; ++l) {
+      e2[l] = A.get(size_t(mp) * lv[l].nr * lv[l].nt * vb);
+      if (!e2[l]) tmp2 = nullptr;
+    }
+    if (!tmp2) cudaGetLastError();
+    plan_tiles();
+  }
   const int nblk = residual_blocks(lv[0].nr, lv[0].nt);
   d_act = static_cast<int*>(A.get(sizeof(int) * mp));
   d_nact = static_cast<int*>(A.get(sizeof(int)));
@@ -452,7 +462,7 @@ void MGSolver::fused(int lo, const VSmemArgs& v, cudaStream_t st) {
     launch_vsmem<double>(v, batch, (const double2*)f[lo], (double2*)e[lo], st);
 }
 void MGSolver::residual(const double2* ff, const double2* u, double tol, cudaStream_t st,
-                        int use_cond, unsigned long long cond) {
+                        int use_cond, unsigned long long cond, int hand_over) {
   RetireArgs ra;
   ra.S = S;
   ra.tol = tol;
@@ -462,7 +472,7 @@ void MGSolver::residual(const double2* ff, const double2* u, double tol, cudaStr
   ra.handle = cond;
   ra.gcnt = d_gcnt;
   ra.zero_guess = zero_guess;
-  ra.tail_planes = tail_planes;
+  ra.tail_planes = hand_over;
   if (opt.precision)
     launch_residual<float>(lv[0], batch, ff, u, (float2*)f[0], d_part, d_psum, d_cnt, ra, st, d_ctab, d_dtab);
   else
@@ -522,6 +532,7 @@ void MGSolver::set_schedule(int nu1, int nu2, int n_sor, Tiles tiles, int nu1f, 
   vs.nu2 = vsb.nu2 = nu2f > 0 ? nu2f : nu2;
   opt.n_sor = vs.n_sor = vsb.n_sor = n_sor;
   opt.tiles = tiles;
+  plan_tiles();
   prepare_tail();
 }
 
@@ -637,8 +648,12 @@ void MGSolver::tail(const double2* ff, double2* u, double tol, cudaStream_t st) 
 void MGSolver::init_loop(cudaStream_t st) { launch_init_active(d_act, d_nact, max_planes, S, st); }
 
 void MGSolver::loop_body(const double2* ff, double2* u, double tol, cudaStream_t st, int use_cond,
-                         unsigned long long cond) {
-  residual(ff, u, tol, st, use_cond, cond);
+                         unsigned long long cond, bool few) {
+  residual(ff, u, tol, st, use_cond, cond, few || !few_phase() ? tail_planes : few_planes);
+  if (few) {
+    vcycle_few(st, u);
+    return;
+  }
   if (vcycle(st, u)) return;
   if (opt.precision)
     launch_update<float>(lv[0], batch, u, (const float2*)e[0], st);
@@ -649,28 +664,97 @@ void MGSolver::loop_body(const double2* ff, double2* u, double tol, cudaStream_t
 int MGSolver::eager_solve(const double2* ff, double2* u, double tol, cudaStream_t st,
                           std::string& err) {
   init_loop(st);
-  for (int it = 0; it <= opt.max_cycles + 1; ++it) {
-    residual(ff, u, tol, st, 0, 0);
-    cudaMemcpyAsync(h_cont, d_cont, sizeof(int), cudaMemcpyDeviceToHost, st);
-    const cudaError_t le = cudaGetLastError();
-    const cudaError_t se = cudaStreamSynchronize(st);
-    if (le != cudaSuccess || se != cudaSuccess) {
-      err = std::string("multigrid iteration: ") + cudaGetErrorString(le != cudaSuccess ? le : se);
-      return -2;
+  for (int phase = many_phase() ? 0 : 1; phase < (few_phase() ? 2 : 1); ++phase) {
+    bool handed = false;
+    for (int it = 0; it <= opt.max_cycles + 1 && !handed; ++it) {
+      residual(ff, u, tol, st, 0, 0, phase == 1 || !few_phase() ? tail_planes : few_planes);
+      cudaMemcpyAsync(h_cont, d_cont, sizeof(int), cudaMemcpyDeviceToHost, st);
+      const cudaError_t le = cudaGetLastError();
+      const cudaError_t se = cudaStreamSynchronize(st);
+      if (le != cudaSuccess || se != cudaSuccess) {
+        err = std::string("multigrid iteration: ") + cudaGetErrorString(le != cudaSuccess ? le : se);
+        return -2;
+      }
+      if (!*h_cont) return 0;
+      if (phase == 1) {
+        vcycle_few(st, u);
+      } else if (!vcycle(st, u)) {
+        if (opt.precision)
+          launch_update<float>(lv[0], batch, u, (const float2*)e[0], st);
+        else
+          launch_update<double>(lv[0], batch, u, (const double2*)e[0], st);
+      }
+      handed = *h_cont == 2;   // few planes remain: the next phase, or the tail kernel, takes them
     }
-    if (!*h_cont) return 0;
-    if (!vcycle(st, u)) {
-      if (opt.precision)
-        launch_update<float>(lv[0], batch, u, (const float2*)e[0], st);
-      else
-        launch_update<double>(lv[0], batch, u, (const double2*)e[0], st);
-    }
-    if (*h_cont == 2) {   // at most tail_planes remain: the tail kernel finishes them
-      tail(ff, u, tol, st);
-      return 0;
-    }
+    if (!handed) return 0;
   }
+  tail(ff, u, tol, st);
   return 0;
+}
+
+// A V-cycle of the last few planes: the window passes above level base.
+void MGSolver::vcycle_few(cudaStream_t st, double2* u) {
+  for (int l = 0; l < base; ++l)
+    for (const TileStep& t : t_down[l]) launch_tile(lv[l], lv[l + 1], batch, t, st);
+  fused(base, vsb, st);
+  for (int l = base - 1; l >= 0; --l)
+    for (TileStep t : t_up[l]) {
+      t.u = u;
+      launch_tile(lv[l], lv[l + 1], batch, t, st);
+    }
+}
+
+// The launches of a smoothing leg of `cycles` cycles on a level, as few as the
+// halos allow; empty when the windows do not take the level or the schedule.
+static std::vector<TileStep> tile_chain(const LevelDev& L, int n_sor, int cycles, int op_first, int op_last,
+                                        const float2* src, float2* dst, float2* x0, float2* x1) {
+  for (int c = cycles; c >= 1; --c) {
+    std::vector<TileStep> out;
+    bool ok = true;
+    for (int done = 0; done < cycles && ok; done += c) {
+      TileStep t{};
+      const int now = std::min(c, cycles - done);
+      const bool last = done + now == cycles;
+      ok = tile_step(L.nr, L.nt, n_sor, now, last && (op_last & TILE_RESTRICT), t);
+      t.op = (done == 0 ? op_first : 0) | (last ? op_last : 0);
+      t.src = done == 0 ? src : out.back().dst;
+      t.dst = last ? dst : (out.size() % 2 == 0 ? x0 : x1);
+      out.push_back(t);
+    }
+    if (ok) return out;
+  }
+  return {};
+}
+
+// The window passes for the current schedule, and the number of planes from
+// which on a solve takes them: as many as two rounds of the chip's windows hold
+// (256 x 128 cells, two cycles a launch: 16 planes of 36 windows).
+void MGSolver::plan_tiles() {
+  few_planes = 0;
+  t_down.clear();
+  t_up.clear();
+  if (!tmp2 || opt.nu1 < 1 || opt.nu2 < 1) return;
+  int planes = max_planes;
+  for (int l = 0; l < base; ++l) {
+    const int nu1 = l >= first ? vs.nu1 : opt.nu1, nu2 = l >= first ? vs.nu2 : opt.nu2;
+    float2* E = static_cast<float2*>(e[l]);
+    float2* T = static_cast<float2*>(tmp);
+    float2* X = static_cast<float2*>(tmp2);
+    std::vector<TileStep> dn = tile_chain(lv[l], opt.n_sor, nu1, 0, TILE_RESTRICT, nullptr, E, T, X);
+    std::vector<TileStep> up = tile_chain(lv[l], opt.n_sor, nu2, TILE_PROLONG, l == 0 ? TILE_UPDATE : 0, E,
+                                          l == 0 ? nullptr : static_cast<float2*>(e2[l]), T, X);
+    if (dn.empty() || up.empty()) return;
+    for (TileStep& t : dn) t.fc = static_cast<float2*>(f[l + 1]);
+    for (TileStep& t : up) t.ec = static_cast<const float2*>(l + 1 >= base ? e[l + 1] : e2[l + 1]);
+    for (std::vector<TileStep>* leg : {&dn, &up})
+      for (TileStep& t : *leg) {
+        t.f = static_cast<const float2*>(f[l]);
+        planes = std::min(planes, std::max(1, 2 * tile_slots(lv[l].nr, lv[l].nt) / (t.ntx * t.nty)));
+      }
+    t_down.push_back(dn);
+    t_up.push_back(up);
+  }
+  few_planes = planes;
 }
 
 }  // namespace ps

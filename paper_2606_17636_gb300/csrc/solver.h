@@ -53,12 +53,18 @@ class MGSolver {
   // mode the host reads the continue flag each iteration.
   void init_loop(cudaStream_t st);
   void loop_body(const double2* f, double2* u, double tol, cudaStream_t st, int use_cond,
-                 unsigned long long cond);
+                 unsigned long long cond, bool few);
+  // A solve's phases: iterations with the level-wide passes while more than
+  // few_planes planes remain (none when the batch is no larger), then
+  // iterations with the window passes.
+  bool many_phase() const { return few_planes < batch.max_planes; }
+  bool few_phase() const { return few_planes > 0; }
   int eager_solve(const double2* f, double2* u, double tol, cudaStream_t st, std::string& err);
   // One V-cycle; with u, the refinement's update u += e rides on the last
   // smoothing pass when the schedule post-smooths level 0 with the
   // level-wide passes (returns true then; else the caller updates).
   bool vcycle(cudaStream_t st, double2* u = nullptr);
+  void vcycle_few(cudaStream_t st, double2* u);
   // Change the smoothing schedule and tile shapes of later V-cycles (a
   // captured solve must be captured again).
   void set_schedule(int nu1, int nu2, int n_sor, Tiles tiles, int nu1f, int nu2f);
@@ -82,6 +88,15 @@ class MGSolver {
   // the level from which a solve's V-cycle runs it, and its arguments there
   int base = 0;
   VSmemArgs vsb{};
+  // window passes (k_tile.cu, mixed path) for the last few_planes planes of a
+  // solve (0: none): per level below base the launches before and after the
+  // coarse correction; e2[l] takes level l's result after it, tmp2 is a second
+  // scratch buffer
+  int few_planes = 0;
+  std::vector<std::vector<TileStep>> t_down, t_up;
+  std::vector<void*> e2;
+  void* tmp2 = nullptr;
+  void plan_tiles();
   int zero_guess = 0;              // the next solve starts from u = 0 (set by the caller)
   VSmemArgs vs{};
   // stage helpers on explicit buffers
@@ -93,8 +108,9 @@ class MGSolver {
   // levels lo .. coarsest in shared memory, with v built for lo
   void fused(int lo, const VSmemArgs& v, cudaStream_t st);
   bool build_vsmem(Arena& A, int lo, int n_modes, VSmemArgs& v, std::string& err);
+  // hand_over: the continue flag becomes 2 once at most that many planes remain
   void residual(const double2* f, const double2* u, double tol, cudaStream_t st, int use_cond,
-                unsigned long long cond);
+                unsigned long long cond, int hand_over);
   // the defect alone into r (tolerance 0: no plane retires)
   void residual_to(const double2* f, const double2* u, void* r, cudaStream_t st);
   int* d_act = nullptr;

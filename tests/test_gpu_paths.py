@@ -53,3 +53,63 @@ def test_fp64_levels_run_level_wide(ps, nr, nt, nu1f, nu2f):
         if not nu1f:
             assert abs(cyc[m] - H.solve(m, b, 1e-12)[1]) <= 1
     s.close()
+
+
+# n_r, n_tz, n_phi, SOR sweeps.  Above 1.5 M cells over all planes lines of 32 to
+# 512 cells are relaxed in registers (16 cells a lane at 512; column tiles of at
+# most 30 pairs a warp; segments of columns); the others, 4 sweeps and lines of
+# 16 cells stay with the staged passes, whose sizes are here too.
+SMOOTH_GRIDS = [(32, 32, 4, 2), (64, 16, 4, 2), (512, 32, 4, 2), (32, 512, 4, 3), (32, 256, 512, 2), (256, 32, 512, 1),
+                (64, 64, 1024, 3), (128, 128, 256, 2), (512, 32, 256, 2), (32, 512, 256, 2), (512, 64, 128, 3), (64, 512, 128, 1),
+                (512, 512, 16, 2), (256, 128, 128, 4)]
+
+
+@pytest.mark.parametrize("nr,nt,n_phi,n_sor", SMOOTH_GRIDS)
+def test_level_wide_smoothing_of_every_line_length(ps, nr, nt, n_phi, n_sor):
+    """Two cycles on the finest level against the oracle's Algorithm 1 in some
+    modes (FP32 rounding through the sweeps: 2e-5 of the largest value, as for
+    the stage tests)."""
+    from oracle import mg
+    sp = workloads.spec(workloads.CYLINDRICAL, nr, nt, n_phi, workloads.UNIFORM, 1.0, 2.0, 0.0, nt / nr)
+    s = ps.Solver.from_spec(sp, precision=ps.MIXED, use_graph=False)
+    s.set_schedule(2, 2, n_sor)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(nr + nt)
+    e0 = torch.randn((s.n_modes, nt, nr), generator=gen, dtype=torch.complex64, device="cuda")
+    f = torch.randn((s.n_modes, nt, nr), generator=gen, dtype=torch.complex64, device="cuda")
+    got = s.stage_smooth(0, e0.clone(), f, 2)
+    H = mg.Hierarchy(oracle_plane(sp), n_sor=n_sor)
+    for m in (0, s.n_modes - 1):
+        u = np.zeros((nr + 2, nt + 2), complex)
+        u[1:-1, 1:-1] = e0[m].cpu().numpy().T
+        H.smooth(0, m, u, f[m].cpu().numpy().T.astype(complex), 2)
+        ref = u[1:-1, 1:-1].T
+        assert np.abs(got[m].cpu().numpy() - ref).max() <= 2e-5 * np.abs(ref).max()
+    s.close()
+
+
+# finest level 256 x 128 (one level above the shared-memory ones) and 512 x 256
+# (two), schedules that need one or several launches a leg or none at all
+FEW = [(256, 128, (2, 1, 2, 3, 1)), (256, 128, (3, 2, 2, 0, 0)), (256, 128, (1, 1, 1, 0, 0)), (256, 128, (2, 2, 3, 0, 0)),
+       (256, 128, (2, 2, 5, 0, 0)), (512, 256, (2, 2, 2, 0, 0)), (256, 256, (2, 1, 2, 0, 0)), (512, 32, (2, 2, 2, 0, 0))]
+
+
+@pytest.mark.parametrize("nr,nt,sched", FEW)
+def test_last_planes_take_the_window_passes_with_the_same_result(ps, nr, nt, sched):
+    """A plane's iteration does not depend on how many others are active: the
+    level-wide passes and, for the last few, the passes on windows give the same
+    bits (mixed path), and the same cycle counts."""
+    sp = workloads.spec(workloads.CYLINDRICAL, nr, nt, 64, workloads.UNIFORM, 1.0, 3.0, 0.0, 2.0 * nt / nr)
+    s = ps.Solver.from_spec(sp, precision=ps.MIXED, use_graph=False)
+    s.set_schedule(*sched[:3], nu_pre_fused=sched[3], nu_post_fused=sched[4])
+    f = torch.from_numpy(_planes((s.n_modes, nt, nr), 5)).cuda()
+    u, cyc, rc = s.stage_mg_solve(f, tol=1e-8)
+    assert rc == ps.OK
+    for modes in ([0], [1, 7, 32]):
+        g = torch.zeros_like(f)
+        g[modes] = f[modes]
+        v, cyc2, rc = s.stage_mg_solve(g, tol=1e-8)
+        assert rc == ps.OK
+        assert torch.equal(v[modes], u[modes]) and [cyc2[m] for m in modes] == [cyc[m] for m in modes]
+        assert torch.count_nonzero(v) == torch.count_nonzero(v[modes])
+    s.close()
