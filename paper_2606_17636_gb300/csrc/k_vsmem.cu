@@ -6,7 +6,8 @@
 // of kernel boundaries.  Input f[first] and output e[first] live in global
 // memory.  The coarsest level is solved directly: in FP64 by the FP64
 // kernel; a separable coarsest level in FP32 by the FP32 kernel, with factors
-// computed in FP64 on the host (coarsest_f32c).
+// computed in FP64 on the host (coarsest_f32c).  An FP32 first level of 4096 or
+// 8192 cells is held in registers instead (k_vpatch, patch.cuh).
 //
 // Shared-memory layout of a level (nr x nt, unpadded rows): cell (j, i) sits
 // at j * nr + (i ^ h(j)).  The row swizzle h(j) < min(16, nr) follows the
@@ -15,10 +16,12 @@
 // pair (16 bytes, one bank group) stay together.  Row-wise vector accesses of
 // radial lines and the column accesses of polar lines (pairs of columns for
 // FP32) are then free of bank conflicts.
+#include <cstdint>
 #include <cstdio>
 #include <type_traits>
 
 #include "lines.cuh"
+#include "patch.cuh"
 
 namespace ps {
 
@@ -591,166 +594,193 @@ __device__ __forceinline__ void ld_kb(float (&w)[KB], const float* p) {
 }
 
 // z = (1/pivot) .* ((V^-1 (x) I) f): each task takes KB eigenvalues k0 .. of
-// one part (mirror-symmetric: sums f_j + f_{nt-1-j} for the even
-// eigenvectors k < nt/2, differences for the odd ones) at one radial index,
-// both components, so every f value it loads feeds 2 KB products.
-template <int KB>
-__device__ void f32c_forward(const LevelDev& Lc, const float2* fc, const float* ViT, const float* invd,
-                             float* z, bool sym) {
-  const int nr = Lc.nr, nt = Lc.nt, P = nr + 1, nc = P * nt, h = nt / 2, vr = sym ? h : nt;
-  const int kper = sym ? h : nt, nkb = kper / KB, ntask = (sym ? 2 : 1) * nr * nkb;
+// one part (SYM: sums f_j + f_{nt-1-j} for the even eigenvectors k < nt/2,
+// differences for the odd ones) at two neighbouring radial indices, both
+// components as packed pairs, so a step's three loads feed 4 KB products.
+// (With one radial index a task the addresses and loads were two thirds of
+// the instructions: 4 100 cycles for 64 x 32 cells, now 2 300.)
+template <int KB, bool SYM>
+__device__ __forceinline__ void f32c_forward(const LevelDev& Lc, const float2* fc, const float* ViT, const float* invd,
+                                             float* z) {
+  const int nr = Lc.nr, nt = Lc.nt, P = nr + 1, nc = P * nt, h = nt / 2, vr = SYM ? h : nt;
+  const int nkb = vr / KB, np = nr / 2, ntask = (SYM ? 2 : 1) * np * nkb;
+  const int mask = (nr < 16 ? nr : 16) - 1, sh = nt > 32 ? 0 : 1;   // the swizzle of vslot
   for (int t = threadIdx.x; t < ntask; t += blockDim.x) {
-    const int i = t % nr, rest = t / nr, kb = rest % nkb, part = rest / nkb;
-    const int k0 = part * h + kb * KB;
-    float ax[KB], ay[KB];
+    const int rest = t / np, i = 2 * (t - rest * np), part = rest >= nkb ? 1 : 0;
+    const int k0 = part * h + (rest - part * nkb) * KB;
+    const float sg = part ? -1.f : 1.f;
+    float2 a[KB], b[KB];
 #pragma unroll
-    for (int q = 0; q < KB; ++q) ax[q] = ay[q] = 0.f;
+    for (int q = 0; q < KB; ++q) a[q] = b[q] = make_float2(0.f, 0.f);
+    auto pair = [&](float2& x, float2& y, int j) {
+      ld_pair(x, y, fc + j * nr + (i ^ ((sh ? 2 * j : j & ~1) & mask)));
+    };
+#pragma unroll 4
     for (int j = 0; j < vr; ++j) {
-      float2 s = fc[vslot<float>(Lc, j, i)];
-      if (sym) {
-        const float2 v = fc[vslot<float>(Lc, nt - 1 - j, i)];
-        s = part ? make_float2(s.x - v.x, s.y - v.y) : make_float2(s.x + v.x, s.y + v.y);
+      float2 x, y;
+      pair(x, y, j);
+      if constexpr (SYM) {
+        float2 u, v;
+        pair(u, v, nt - 1 - j);
+        x = fma2(sg, u, x);   // exactly the sum or difference
+        y = fma2(sg, v, y);
       }
       float w[KB];
       ld_kb<KB>(w, ViT + j * nt + k0);
 #pragma unroll
       for (int q = 0; q < KB; ++q) {
-        ax[q] = fmaf(w[q], s.x, ax[q]);
-        ay[q] = fmaf(w[q], s.y, ay[q]);
+        a[q] = fma2(w[q], x, a[q]);
+        b[q] = fma2(w[q], y, b[q]);
       }
     }
 #pragma unroll
     for (int q = 0; q < KB; ++q) {
-      const int k = k0 + q;
-      const float d = invd[k * P + i];
-      z[k * P + i] = ax[q] * d;
-      z[nc + k * P + i] = ay[q] * d;
+      const int o = (k0 + q) * P + i;
+      const float d = invd[o], e = invd[o + 1];
+      z[o] = a[q].x * d;
+      z[o + 1] = b[q].x * e;
+      z[nc + o] = a[q].y * d;
+      z[nc + o + 1] = b[q].y * e;
     }
   }
 }
 
-// e = (V (x) I) x: each task takes JB rows j0 .. (mirror-symmetric: j < nt/2,
-// writing e_j = E + O and e_{nt-1-j} = E - O from the even and odd
-// eigenvector parts) at one radial index, both components.
-template <int JB>
-__device__ void f32c_back(const LevelDev& Lc, const float* z, const float* VT, float2* ec, bool sym) {
-  const int nr = Lc.nr, nt = Lc.nt, P = nr + 1, nc = P * nt, h = nt / 2, vr = sym ? h : nt;
+// e = (V (x) I) x: each task takes JB rows j0 .. (SYM: j < nt/2, writing
+// e_j = E + O and e_{nt-1-j} = E - O from the even and odd eigenvector
+// parts) at one radial index, both components as a packed pair (2 050 cycles
+// for 64 x 32 cells; 3 600 with the factors behind a generic pointer and 4
+// steps' loads in flight).
+template <int JB, bool SYM>
+__device__ __forceinline__ void f32c_back(const LevelDev& Lc, const float* z, const float* VT, float2* ec) {
+  const int nr = Lc.nr, nt = Lc.nt, P = nr + 1, nc = P * nt, h = nt / 2, vr = SYM ? h : nt;
   const int njb = vr / JB, ntask = nr * njb;
   for (int t = threadIdx.x; t < ntask; t += blockDim.x) {
-    const int i = t % nr, j0 = (t / nr) * JB;
-    float ex[JB], ey[JB], ox[JB], oy[JB];
+    const int jb = t / nr, i = t - jb * nr, j0 = jb * JB;
+    float2 E[JB], O[JB];
 #pragma unroll
-    for (int q = 0; q < JB; ++q) ex[q] = ey[q] = ox[q] = oy[q] = 0.f;
-    const int ke = sym ? h : nt;
-    for (int k = 0; k < ke; ++k) {
-      const float xr = z[k * P + i], xi = z[nc + k * P + i];
+    for (int q = 0; q < JB; ++q) E[q] = O[q] = make_float2(0.f, 0.f);
+    const float *zr = z + i, *zi = zr + nc, *vt = VT + j0;
+#pragma unroll 8
+    for (int k = 0; k < vr; ++k) {
       float w[JB];
-      ld_kb<JB>(w, VT + k * vr + j0);
+      ld_kb<JB>(w, vt + k * vr);
+      const float2 x = make_float2(zr[k * P], zi[k * P]);
 #pragma unroll
-      for (int q = 0; q < JB; ++q) {
-        ex[q] = fmaf(w[q], xr, ex[q]);
-        ey[q] = fmaf(w[q], xi, ey[q]);
-      }
-    }
-    if (sym) {
-      for (int k = h; k < nt; ++k) {
-        const float xr = z[k * P + i], xi = z[nc + k * P + i];
-        float w[JB];
-        ld_kb<JB>(w, VT + k * vr + j0);
+      for (int q = 0; q < JB; ++q) E[q] = fma2(w[q], x, E[q]);
+      if constexpr (SYM) {
+        ld_kb<JB>(w, vt + (k + h) * vr);
+        const float2 y = make_float2(zr[(k + h) * P], zi[(k + h) * P]);
 #pragma unroll
-        for (int q = 0; q < JB; ++q) {
-          ox[q] = fmaf(w[q], xr, ox[q]);
-          oy[q] = fmaf(w[q], xi, oy[q]);
-        }
+        for (int q = 0; q < JB; ++q) O[q] = fma2(w[q], y, O[q]);
       }
     }
 #pragma unroll
     for (int q = 0; q < JB; ++q) {
       const int j = j0 + q;
-      ec[vslot<float>(Lc, j, i)] = make_float2(ex[q] + ox[q], ey[q] + oy[q]);
-      if (sym) ec[vslot<float>(Lc, nt - 1 - j, i)] = make_float2(ex[q] - ox[q], ey[q] - oy[q]);
+      ec[vslot<float>(Lc, j, i)] = make_float2(E[q].x + O[q].x, E[q].y + O[q].y);
+      if constexpr (SYM) ec[vslot<float>(Lc, nt - 1 - j, i)] = make_float2(E[q].x - O[q].x, E[q].y - O[q].y);
     }
   }
 }
 
+// d_i <- d_i + m_i d_{i-1} (UP; else the entry after) along a line of which each of S
+// neighbouring lanes holds 8 entries (S a power of two, at most 32; lane seg
+// of them; m is zero at the line's first entry).
+template <bool UP>
+__device__ __forceinline__ void scan8(float (&d)[8], float (&m)[8], int seg, int S) {
+#pragma unroll
+  for (int s = 1; s < 8; ++s) {   // from a zero start; m becomes the factor of the carry
+    const int i = UP ? s : 7 - s, b = UP ? i - 1 : i + 1;
+    d[i] = fmaf(m[i], d[b], d[i]);
+    m[i] *= m[b];
+  }
+  float D = d[UP ? 7 : 0], M = m[UP ? 7 : 0];
+  for (int o = 1; o < S; o *= 2) {
+    const float x = UP ? __shfl_up_sync(0xffffffffu, D, o) : __shfl_down_sync(0xffffffffu, D, o);
+    const float y = UP ? __shfl_up_sync(0xffffffffu, M, o) : __shfl_down_sync(0xffffffffu, M, o);
+    if (UP ? seg >= o : seg + o < S) {
+      D = fmaf(M, x, D);
+      M *= y;
+    }
+  }
+  float x = UP ? __shfl_up_sync(0xffffffffu, D, 1) : __shfl_down_sync(0xffffffffu, D, 1);
+  if (seg == (UP ? 0 : S - 1)) x = 0.f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) d[i] = fmaf(m[i], x, d[i]);
+}
+
 // e = L_m^-1 f on the coarsest level Lc (cells in the FP32 swizzled layout);
 // scratch z [2][nt][nr + 1] FP32 at dbl_off.
-__device__ void coarsest_f32c(const VSmemArgs& a, int slot, unsigned char* vraw, const LevelDev& Lc,
-                              const float2* fc, float2* ec) {
+template <bool SM, bool SYM>   // factors in shared memory; mirror-symmetric form
+__device__ __forceinline__ void coarsest_f32c(const VSmemArgs& a, int slot, unsigned char* vraw, const LevelDev& Lc,
+                                              const float2* fc, float2* ec) {
   const int nr = Lc.nr, nt = Lc.nt, P = nr + 1, nc = P * nt;
-  const bool sym = a.sep_sym != 0;
-  const int vr = sym ? nt / 2 : nt;
+  const int vr = SYM ? nt / 2 : nt;
   float* z = reinterpret_cast<float*>(vraw + a.dbl_off);
-  const float* ViT = a.blk_smem ? reinterpret_cast<const float*>(vraw + a.blk_off)
-                                : a.sepf + size_t(slot) * a.sepf_stride;
+  const float* ViT;
+  if constexpr (SM) ViT = reinterpret_cast<const float*>(vraw + a.blk_off);
+  else ViT = a.sepf + size_t(slot) * a.sepf_stride;
   const float* VT = ViT + vr * nt;
   const float* invd = VT + nt * vr;
   const float* cp = invd + nc;
   const float* lid = cp + nc;
-  if (vr % 4 == 0) f32c_forward<4>(Lc, fc, ViT, invd, z, sym);
-  else f32c_forward<1>(Lc, fc, ViT, invd, z, sym);
+  if (vr % 4 == 0) f32c_forward<4, SYM>(Lc, fc, ViT, invd, z);
+  else f32c_forward<1, SYM>(Lc, fc, ViT, invd, z);
   __syncthreads();
-  // Thomas sweeps per (component, eigenvalue), one FMA per step each way:
-  // dp_i = z_i - lid_i dp_{i-1}, then x_i = dp_i - cp_i x_{i+1}, in place;
-  // the 2 nt systems on the first four warps
-  {
-    const int nsys = 2 * nt, per = (nsys + 3) / 4;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp < 4 && lane < per && warp * per + lane < nsys) {
-      const int q = warp * per + lane, c = q / nt, k = q - c * nt;
-      float* __restrict__ zz = z + c * nc + k * P;
-      const float* __restrict__ lk = lid + k * P;
-      const float* __restrict__ ck = cp + k * P;
-      // in batches of eight steps: the loads of a batch are issued together,
-      // so one shared-memory latency is paid per batch, not per step
-      float dp = zz[0];
-      int i = 1;
-      for (; i + 8 <= nr; i += 8) {
-        float zv[8], lv[8];
+  // Radial solves per (component, eigenvalue): dp_i = z_i - lid_i dp_{i-1},
+  // then x_i = dp_i - cp_i x_{i+1}, in place.  A thread takes a segment of 8
+  // entries from a zero start and the factor by which a carry passes through
+  // each entry; the carries meet by a scan over the nr / 8 neighbouring lanes.
+  // (One thread per system, 63 dependent steps each way for 64 x 32 cells:
+  // 3 400 cycles; the scan: 1 900.)
+  if (nr >= 8 && nr <= 256 && (nr & (nr - 1)) == 0) {
+    const int S = nr / 8, tasks = 2 * nt * S;
+    for (int t0 = 0; t0 < tasks; t0 += blockDim.x) {
+      const int t = t0 + threadIdx.x, seg = t & (S - 1);
+      const bool on = t < tasks;
+      const int q = on ? t / S : 0, k = q >= nt ? q - nt : q;
+      float* zz = z + (q >= nt ? nc : 0) + k * P + 8 * seg;
+      const float* lk = lid + k * P + 8 * seg;
+      const float* ck = cp + k * P + 8 * seg;
+      float d[8], l[8], c[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          zv[q] = zz[i + q];
-          lv[q] = lk[i + q];
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          dp = fmaf(-lv[q], dp, zv[q]);
-          zv[q] = dp;
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q) zz[i + q] = zv[q];
+      for (int i = 0; i < 8; ++i) {
+        d[i] = zz[i];
+        l[i] = -lk[i];
+        c[i] = -ck[i];
       }
-      for (; i < nr; ++i) {
-        dp = fmaf(-lk[i], dp, zz[i]);
-        zz[i] = dp;
-      }
-      float xv = dp;
-      i = nr - 2;
-      for (; i >= 7; i -= 8) {
-        float zv[8], cv[8];
+      if (seg == 0) l[0] = 0.f;
+      if (seg == S - 1) c[7] = 0.f;
+      scan8<true>(d, l, seg, S);
+      scan8<false>(d, c, seg, S);
+      if (on) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          zv[q] = zz[i - q];
-          cv[q] = ck[i - q];
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          xv = fmaf(-cv[q], xv, zv[q]);
-          zv[q] = xv;
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q) zz[i - q] = zv[q];
+        for (int i = 0; i < 8; ++i) zz[i] = d[i];
       }
-      for (; i >= 0; --i) {
-        xv = fmaf(-ck[i], xv, zz[i]);
-        zz[i] = xv;
-      }
+    }
+  } else {   // one thread per system
+    for (int q = threadIdx.x; q < 2 * nt; q += blockDim.x) {
+      const int k = q >= nt ? q - nt : q;
+      float* zz = z + (q >= nt ? nc : 0) + k * P;
+      float v = zz[0];
+      for (int i = 1; i < nr; ++i) zz[i] = v = fmaf(-lid[k * P + i], v, zz[i]);
+      for (int i = nr - 2; i >= 0; --i) zz[i] = v = fmaf(-cp[k * P + i], v, zz[i]);
     }
   }
   __syncthreads();
-  if (vr % 4 == 0) f32c_back<4>(Lc, z, VT, ec, sym);
-  else f32c_back<1>(Lc, z, VT, ec, sym);
+  if (vr % 4 == 0) f32c_back<4, SYM>(Lc, z, VT, ec);
+  else f32c_back<1, SYM>(Lc, z, VT, ec);
   __syncthreads();
+}
+__device__ __forceinline__ void coarsest_f32c(const VSmemArgs& a, int slot, unsigned char* vraw, const LevelDev& Lc,
+                                              const float2* fc, float2* ec) {
+  if (a.blk_smem) {
+    if (a.sep_sym) coarsest_f32c<true, true>(a, slot, vraw, Lc, fc, ec);
+    else coarsest_f32c<true, false>(a, slot, vraw, Lc, fc, ec);
+  } else {
+    if (a.sep_sym) coarsest_f32c<false, true>(a, slot, vraw, Lc, fc, ec);
+    else coarsest_f32c<false, false>(a, slot, vraw, Lc, fc, ec);
+  }
 }
 
 // The first fused level's right-hand side from global memory (this plane's
@@ -772,6 +802,37 @@ __device__ __forceinline__ void stage_f0(const VSmemArgs& a, vec2_t<T>* sm, cons
   }
 }
 
+// Every level's coefficient tables and this mode's omega rows into shared
+// memory (asynchronous copies to tb, after the error / right-hand-side arrays), and
+// block-local level descriptors that point at them.  One flat copy of this
+// slot's packed tables: each level's block starts one element past an even
+// element offset, so the two entries of a cell pair are one aligned vector load.
+template <typename T>
+__device__ __forceinline__ void stage_tables(const VSmemArgs& a, int slot, T* tb, LevelDev* sL) {
+  typedef typename std::conditional<sizeof(T) == 4, float4, double2>::type W4;
+  constexpr int per = int(sizeof(W4) / sizeof(T));
+  const W4* src = reinterpret_cast<const W4*>(static_cast<const T*>(a.tabs) + size_t(slot) * a.tab_stride);
+  W4* dst = reinterpret_cast<W4*>(tb);
+  for (int k = threadIdx.x; k < a.tab_stride / per; k += blockDim.x) cp_async_v(dst + k, src + k, true);
+  if (threadIdx.x == 0) {
+    int toff = 0;
+    for (int l = 0; l < a.nlev; ++l) {
+      const LevelDev& G = a.L[l];
+      const int NR = G.nr + 2, NT = G.nt + 2;
+      toff = (toff + 1) / 2 * 2 + 1;
+      T* srt = tb + toff;
+      T* stt = srt + RT_N * NR;
+      T* sor = stt + TT_N * NT;
+      T* sot = sor + G.nt;
+      LevelDev d = G;
+      if constexpr (sizeof(T) == 8) { d.rd = srt; d.td = stt; d.omr_d = sor; d.omt_d = sot; }
+      else { d.rf = srt; d.tf = stt; d.omr_f = sor; d.omt_f = sot; }
+      sL[l] = d;
+      toff += RT_N * NR + TT_N * NT + G.nt + G.nr;
+    }
+  }
+}
+
 template <typename T, int NTH>
 __global__ void __launch_bounds__(NTH, 1) k_vsmem(VSmemArgs a, Batch B, const vec2_t<T>* __restrict__ gf,
                                                vec2_t<T>* __restrict__ ge) {
@@ -786,40 +847,8 @@ __global__ void __launch_bounds__(NTH, 1) k_vsmem(VSmemArgs a, Batch B, const ve
   if constexpr (sizeof(T) == 8) s2 = B.s2d[slot]; else s2 = B.s2f[slot];
   const int K = a.nlev;
   const int nr0 = a.L[0].nr, n0 = nr0 * a.L[0].nt;
-  // stage every level's coefficient tables and this mode's omega rows in
-  // shared memory (after the error / right-hand-side arrays) and point a
-  // block-local copy of the level descriptors at them
   __shared__ LevelDev sL[8];
-  {
-    // one flat copy of this slot's packed tables (each level's block starts
-    // one element past an even element offset, so the two entries of a cell
-    // pair are one aligned vector load), then block-local level descriptors
-    T* tb = reinterpret_cast<T*>(sm + a.tab_off);
-    {
-      typedef typename std::conditional<sizeof(T) == 4, float4, double2>::type W4;
-      constexpr int per = int(sizeof(W4) / sizeof(T));
-      const W4* src = reinterpret_cast<const W4*>(static_cast<const T*>(a.tabs) + size_t(slot) * a.tab_stride);
-      W4* dst = reinterpret_cast<W4*>(tb);
-      for (int k = threadIdx.x; k < a.tab_stride / per; k += blockDim.x) cp_async_v(dst + k, src + k, true);
-    }
-    if (threadIdx.x == 0) {
-      int toff = 0;
-      for (int l = 0; l < K; ++l) {
-        const LevelDev& G = a.L[l];
-        const int NR = G.nr + 2, NT = G.nt + 2;
-        toff = (toff + 1) / 2 * 2 + 1;
-        T* srt = tb + toff;
-        T* stt = srt + RT_N * NR;
-        T* sor = stt + TT_N * NT;
-        T* sot = sor + G.nt;
-        LevelDev d = G;
-        if constexpr (sizeof(T) == 8) { d.rd = srt; d.td = stt; d.omr_d = sor; d.omt_d = sot; }
-        else { d.rf = srt; d.tf = stt; d.omr_f = sor; d.omt_f = sot; }
-        sL[l] = d;
-        toff += RT_N * NR + TT_N * NT + G.nt + G.nr;
-      }
-    }
-  }
+  stage_tables<T>(a, slot, reinterpret_cast<T*>(sm + a.tab_off), sL);
   // this mode's coarsest-level factors (when they fit)
   const size_t blk_stride = size_t(a.blk_nt) * a.blk_n * (a.blk_n + 2);
   const size_t fac_stride = a.sep_stride > 0 ? size_t(a.sep_stride) : blk_stride;
@@ -1096,12 +1125,138 @@ __global__ void __launch_bounds__(NTH, 1) k_vsmem(VSmemArgs a, Batch B, const ve
   }
 }
 
+// The same V-cycle with the first level's error in registers (patch.cuh); the
+// levels below and the coarsest solve as in k_vsmem, meanwhile the error waits
+// in its level's shared-memory space.
+template <int PR>
+__global__ void __launch_bounds__(kPatchThreads, 1) k_vpatch(VSmemArgs a, Batch B, const float2* __restrict__ gf,
+                                                              float2* __restrict__ ge) {
+  extern __shared__ __align__(16) unsigned char vraw[];
+  float2* sm = reinterpret_cast<float2*>(vraw);
+  const int nact = *B.nact, p = B.act[blockIdx.x];   // one round trip: the list has an entry per plane
+  if (blockIdx.x >= nact) return;
+  const int slot = B.slot ? B.slot[p] : p;
+  const int m = B.mode[slot];
+  const float s2 = B.s2f[slot];
+  const int K = a.nlev, tid = threadIdx.x;
+  __shared__ LevelDev sL[8];
+  const LevelDev &L0 = a.L[0], &L1 = a.L[1];
+  const int nr = L0.nr, lpr = nr / 4;
+  // this thread's patch in the plane: its rows are whole 32-byte runs
+  const size_t cell = size_t(p) * nr * L0.nt + size_t(PR * (tid / lpr)) * nr + 4 * (tid & (lpr - 1));
+  float2 g[PR][4];
+#pragma unroll
+  for (int r = 0; r < PR; ++r) ld_run(g[r], gf + cell + size_t(r) * nr);
+  float* tab = reinterpret_cast<float*>(sm + a.tab_off);
+  stage_tables<float>(a, slot, tab, sL);
+  if (a.blk_smem && !a.restage) stage_f32c(a, slot, vraw);
+  for (int l = 1; l < K - 1; ++l)
+    for (int k = tid; k < a.L[l].nr * a.L[l].nt; k += kPatchThreads) sm[a.off_e[l] + k] = make_float2(0.f, 0.f);
+  float2* space = sm + a.off_e[0];
+  // the diagonal behind the exchanged rows (32 KB; PR = 2 has its own space)
+  Patch<PR> x(L0, s2, tab + 1, sm + a.off_f[0], space, PR == 2 ? reinterpret_cast<float2*>(vraw + a.dia_off) : space + 8 * kPatchThreads);
+#pragma unroll
+  for (int r = 0; r < PR; ++r) {
+    x.st_f(g[r], r);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) x.E[r][c] = make_float2(0.f, 0.f);
+  }
+  float4* keep = reinterpret_cast<float4*>(space) + tid;
+  auto slot1 = [&](int j, int i) { return vslot<float>(L1, j, i); };
+  cp_async_wait_all();
+  __syncthreads();
+  x.coefficients();
+#pragma unroll 1
+  for (int leg = 0; leg < 2; ++leg) {
+    if (leg) {
+#pragma unroll
+      for (int r = 0; r < PR; ++r)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) keep[(2 * r + h) * kPatchThreads] = x.half(x.E[r], h);
+      for (int l = 1; l < K - 1; ++l) {
+        const LevelDev Lf = sL[l], Lq = sL[l + 1];
+        s_smooth<float>(Lf, sm + a.off_e[l], sm + a.off_f[l], s2, a.nu1, a.n_sor);
+        s_restrict_f32(Lf, Lq, sm + a.off_e[l], sm + a.off_f[l], sm + a.off_f[l + 1], s2);
+      }
+      if (a.restage) {   // the factors take the first level's right-hand side space
+        stage_f32c(a, slot, vraw);
+        cp_async_wait_all();
+        __syncthreads();
+      }
+      coarsest_f32c(a, slot, vraw, a.L[K - 1], sm + a.off_f[K - 1], sm + a.off_e[K - 1]);
+      for (int l = K - 2; l >= 1; --l) {
+        const LevelDev Lf = sL[l], Lq = sL[l + 1];
+        s_prolong_f32(Lf, Lq, sm + a.off_e[l], sm + a.off_e[l + 1], m);
+        s_smooth<float>(Lf, sm + a.off_e[l], sm + a.off_f[l], s2, a.nu2, a.n_sor);
+      }
+      if (a.restage) {
+#pragma unroll
+        for (int r = 0; r < PR; ++r) {
+          ld_run(g[r], gf + cell + size_t(r) * nr);
+          x.st_f(g[r], r);
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < PR; ++r) x.join(x.E[r], keep[2 * r * kPatchThreads], keep[(2 * r + 1) * kPatchThreads]);
+      x.coefficients();
+      x.prolong_from(L1, sm + a.off_e[1], (m & 1) != 0, slot1);
+      __syncthreads();       // every patch is out of the space that the rows take
+    }
+    x.set_dia();
+    x.put(x.bot, 0, PR - 1);
+    x.put(x.bot, 1, PR - 1);
+    const int cycles = leg ? a.nu2 : a.nu1;
+#pragma unroll 1
+    for (int c = 0; c < cycles; ++c) {
+      x.radial(a.n_sor);
+      x.polar(a.n_sor);
+    }
+    if (!leg) {
+      __syncthreads();
+      x.restrict_to(sm + a.off_f[1], slot1);
+      __syncthreads();
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < PR; ++r) st_run(ge + cell + size_t(r) * nr, x.E[r]);
+}
+
+// Rows per patch when the first level's error fits the registers of 512
+// threads (patch.cuh has the times of both kernels), else 0: other sizes, the
+// block or dense coarsest solve, planes that do not start on 32 bytes.
+static int patch_rows(const VSmemArgs& a, const void* gf, const void* ge) {
+  if ((reinterpret_cast<uintptr_t>(gf) | reinterpret_cast<uintptr_t>(ge)) & 31) return 0;   // 32-byte runs
+  const int nr = a.L[0].nr, nt = a.L[0].nt;
+  if (!a.f32c || a.nlev < 2 || nr < 16 || nr > 128 || (nr & (nr - 1))) return 0;
+  if (2 * a.L[1].nr != nr || 2 * a.L[1].nt != nt) return 0;
+  if (nr * nt == 16 * kPatchThreads) return 4;
+  if (nr * nt == 8 * kPatchThreads && a.dia_off) return 2;
+  return 0;
+}
+
+template <int PR>
+static void vpatch(const VSmemArgs& a, const Batch& B, const float2* gf, float2* ge, cudaStream_t st) {
+  static bool attr = false;
+  if (!attr) {
+    cudaFuncAttributes fa;
+    if (cudaFuncGetAttributes(&fa, k_vpatch<PR>) == cudaSuccess)
+      cudaFuncSetAttribute(k_vpatch<PR>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(227 * 1024 - fa.sharedSizeBytes));
+    attr = true;
+  }
+  k_vpatch<PR><<<B.max_planes, kPatchThreads, a.smem_bytes, st>>>(a, B, gf, ge);
+}
+
 // 512 threads (up to 128 registers each, no spills); each warp takes every
 // 16th line of a colour.
 template <typename T>
 void launch_vsmem(const VSmemArgs& a, const Batch& B, const vec2_t<T>* gf, vec2_t<T>* ge,
                   cudaStream_t st) {
   constexpr int NTH = 512;
+  if constexpr (sizeof(T) == 4) {
+    const int pr = patch_rows(a, gf, ge);
+    if (pr == 4) return vpatch<4>(a, B, gf, ge, st);
+    if (pr == 2) return vpatch<2>(a, B, gf, ge, st);
+  }
   static bool attr = false;
   if (!attr) {   // opt in to the largest dynamic size the kernel's static usage leaves
     cudaFuncAttributes fa;

@@ -286,6 +286,7 @@ struct VSmemArgs {
   int blk_n, blk_nt;     // block size (= coarsest nr) and block count (= coarsest nt)
   int blk_smem;          // 1: this slot's factors are staged in shared memory at blk_off
   int dbl_off, blk_off;  // byte offsets in shared memory: FP64 solve scratch, staged factors
+  int dia_off;           // byte offset of the first level's FP32 inverse diagonal (0: no space, see patch.cuh)
   const double* sep;     // separable coarsest-level factors [slots][sep_stride] (sep_stride > 0)
   int sep_stride;
   int sep_sym;           // mirror-symmetric separable layout (see Hierarchy::sep_sym)

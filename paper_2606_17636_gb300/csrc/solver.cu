@@ -201,6 +201,15 @@ bool MGSolver::build_vsmem(Arena& A, int lo, int n_modes, VSmemArgs& v, std::str
   } else if (v.blk_smem) {
     sbytes += blk_bytes;
   }
+  v.dia_off = 0;   // patches of two rows keep the inverse diagonal apart (patch.cuh)
+  const size_t cells0 = size_t(v.L[0].nr) * v.L[0].nt;
+  if (f32c && v.nlev >= 2 && cells0 == 4096) {
+    const size_t at = (sbytes + 15) / 16 * 16;
+    if (at + 4 * cells0 <= 224 * 1024) {
+      v.dia_off = int(at);
+      sbytes = at + 4 * cells0;
+    }
+  }
   v.smem_bytes = sbytes + 16;
   if (H.nc < 16 || (H.nc & (H.nc - 1))) { err = "coarsest level must have a power-of-two size >= 16"; return false; }
   v.nu1 = opt.nu1;

@@ -113,3 +113,42 @@ def test_last_planes_take_the_window_passes_with_the_same_result(ps, nr, nt, sch
         assert torch.equal(v[modes], u[modes]) and [cyc2[m] for m in modes] == [cyc[m] for m in modes]
         assert torch.count_nonzero(v) == torch.count_nonzero(v[modes])
     s.close()
+
+
+# n_r, n_tz, large coarsest level, smoothing counts, SOR sweeps, whole polar
+# range: the first fused level as patches of 4 rows (8192 cells) and of 2
+# (4096 cells), a level below it, both forms of the coarsest solve, factors
+# beside the levels and over the right-hand side
+PATCH_GRIDS = [(256, 128, True, 2, 2, 2, True), (128, 64, True, 1, 1, 2, True), (64, 128, True, 3, 1, 1, True),
+               (128, 64, True, 2, 1, 2, False), (128, 32, True, 2, 2, 3, True), (64, 64, False, 1, 2, 2, True),
+               (32, 128, False, 2, 2, 2, True), (128, 64, False, 2, 2, 2, True), (16, 256, False, 2, 2, 2, True)]
+
+
+@pytest.mark.parametrize("nr,nt,large,nu1,nu2,n_sor,whole", PATCH_GRIDS)
+def test_fused_first_level_held_in_registers(ps, nr, nt, large, nu1, nu2, n_sor, whole):
+    """The fused V-cycle against the oracle's (1e-4, the bound of the V-cycle's
+    stage test), and bitwise against the general kernel, which takes
+    right-hand sides that do not start on a 32-byte boundary."""
+    from oracle import mg
+    sp = workloads.spec(workloads.SPHERICAL, nr, nt, 8, workloads.UNIFORM, 1.0, 2.0,
+                        *(() if whole else (0.3 * np.pi, 0.65 * np.pi)))
+    s = ps.Solver.from_spec(sp, precision=ps.MIXED, use_graph=False,
+                            coarsest_size=ps.COARSEST_LARGE if large else ps.COARSEST_SMALL)
+    s.set_schedule(nu1, nu2, n_sor)
+    lev = s.fused_level()
+    shape = (s.n_modes, nt >> lev, nr >> lev)
+    f = torch.from_numpy(_planes(shape, nr + nt)).to(torch.complex64).cuda()
+    got = s.stage_vcycle(f)
+    room = torch.zeros(f.numel() + 2, dtype=f.dtype, device="cuda")
+    shifted = room[2:].view(shape)
+    shifted.copy_(f)
+    assert f.data_ptr() % 32 == 0 and shifted.data_ptr() % 32 == 16
+    assert torch.equal(got, s.stage_vcycle(shifted))
+    H = mg.Hierarchy(oracle_plane(sp), nu1=nu1, nu2=nu2, n_sor=n_sor,
+                     **(dict(min_cells=32, max_coarse=2048) if large else {}))
+    for m in (0, s.n_modes - 1):
+        u = np.zeros((shape[2] + 2, shape[1] + 2), complex)
+        H.vcycle(lev, m, u, f[m].cpu().numpy().T.astype(complex))
+        ref = u[1:-1, 1:-1].T
+        assert np.abs(got[m].cpu().numpy() - ref).max() <= 1e-4 * np.abs(ref).max()
+    s.close()
