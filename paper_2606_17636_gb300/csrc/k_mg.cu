@@ -6,6 +6,7 @@
 // face of zero area has a zero coefficient, so pole / axis ghosts never enter
 // the stencil.
 #include <cstdio>
+#include <type_traits>
 
 #include "lines.cuh"
 
@@ -253,9 +254,15 @@ int residual_blocks(int nr, int nt) {
   return (nr * nt + 255) / 256;
 }
 
+// What the retirement reads of thread k's plane, loaded ahead (n = 0: not).
+struct RetireHint {
+  int n, iter, p;
+  double2 nf, prev;
+  double fmax2;
+};
 __device__ void retire_block(int* act, int* nact, const Sum4* __restrict__ psum, RetireState S,
                              double tol, int max_cycles, int stagnation, int use_cond,
-                             unsigned long long handle, int* scan, int tail_planes);
+                             unsigned long long handle, int* scan, int tail_planes, const RetireHint& hint);
 
 // FP64 defect at (i, j) from the per-cell products (one FP64 operation for
 // the mode's diagonal read from its own table dm, five fused multiply-adds per
@@ -311,11 +318,30 @@ __device__ __forceinline__ SqPart sq_block_tail(const SqPart* sh, int lane, int 
   return sq_warp_sum4(lane < nw ? sh[lane] : sq_part_zero());
 }
 
+__device__ __forceinline__ void merge_part(SqPart& t, const SqPart* q) {
+  const float4 qs = __ldcg(reinterpret_cast<const float4*>(q->s));
+  const int4 qb = __ldcg(reinterpret_cast<const int4*>(q->e));
+  const float vs[4] = {qs.x, qs.y, qs.z, qs.w};
+  const int vb[4] = {qb.x, qb.y, qb.z, qb.w};
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const SqAcc m = sq_merge(SqAcc{t.s[c], t.e[c]}, SqAcc{vs[c], vb[c]});
+    t.s[c] = m.s;
+    t.e[c] = m.e;
+  }
+}
+__device__ __forceinline__ Sum4 sum_of(const SqPart& q) {
+  return sum4(sq_value(SqAcc{q.s[0], q.e[0]}), sq_value(SqAcc{q.s[1], q.e[1]}), sq_value(SqAcc{q.s[2], q.e[2]}),
+              sq_value(SqAcc{q.s[3], q.e[3]}));
+}
+
+constexpr int kFlatItems = 256;
+
 // The residual work items of one launch.  ZERO: u = 0 on the first
 // iteration, so r = f and |r|^2 = |f|^2 (no stencil); CPT: cells per thread
 // and work item.  Both are fixed per launch, so each combination is its own
 // loop and no branch of the other remains in the cell loop.
-template <typename T, bool ZERO, int CPT>
+template <typename T, bool ZERO, int CPT, bool FLAT>
 __device__ __forceinline__ void residual_items(const LevelDev& L, const Batch& B,
                                                const double2* __restrict__ f,
                                                const double2* __restrict__ u,
@@ -356,6 +382,11 @@ __device__ __forceinline__ void residual_items(const LevelDev& L, const Batch& B
         }
       }
     }
+    RetireHint hint{};   // FLAT: what the retirement will read, in flight during the reduction
+    if (FLAT && !want_f) {
+      const int q = B.act[min(int(threadIdx.x), nact - 1)];
+      hint = RetireHint{nact, *ra.S.iter, q, ra.S.nf2[q], ra.S.nr2[q], *ra.S.fmax2};
+    }
     ax = sq_warp_sum(ax);
     ay = sq_warp_sum(ay);
     if (ZERO) {   // r = f: the same sums
@@ -372,34 +403,34 @@ __device__ __forceinline__ void residual_items(const LevelDev& L, const Batch& B
       if (lane == 0) {
         part[size_t(p) * bpp + bx] = t;
         __threadfence();
-        flag[0] = (atomicAdd(&cnt[p], 1) == ipp - 1);
+        flag[0] = FLAT ? atomicAdd(ra.gcnt, 1) == nact * ipp - 1 : atomicAdd(&cnt[p], 1) == ipp - 1;
       }
     }
     __syncthreads();
-    if (flag[0]) {   // the plane's last item: its sums over the items in item order
+    if (FLAT && flag[0]) {   // the last item of all: a warp per plane, then the retirement
+      __threadfence();
+      for (int kk = warp; kk < nact; kk += nw) {
+        const int pp = B.act[kk];
+        SqPart t = sq_part_zero();
+        for (int b = lane; b < ipp; b += 32) merge_part(t, &part[size_t(pp) * bpp + b]);
+        t = sq_warp_sum4(t);
+        if (lane == 0) psum[pp] = sum_of(t);
+      }
+      __syncthreads();
+      retire_block(const_cast<int*>(B.act), const_cast<int*>(B.nact), psum, ra.S, ra.tol, ra.max_cycles, ra.stagnation,
+                   ra.use_cond, ra.handle, scan, ra.tail_planes, hint);
+      if (threadIdx.x == 0) *ra.gcnt = 0;
+    } else if (flag[0]) {   // the plane's last item: its sums over the items in item order
       __threadfence();
       SqPart t = sq_part_zero();
-      for (int b = threadIdx.x; b < ipp; b += blockDim.x) {
-        const SqPart* q = &part[size_t(p) * bpp + b];
-        const float4 qs = __ldcg(reinterpret_cast<const float4*>(q->s));
-        const int4 qb = __ldcg(reinterpret_cast<const int4*>(q->e));
-        const float vs[4] = {qs.x, qs.y, qs.z, qs.w};
-        const int vb[4] = {qb.x, qb.y, qb.z, qb.w};
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const SqAcc m = sq_merge(SqAcc{t.s[c], t.e[c]}, SqAcc{vs[c], vb[c]});
-          t.s[c] = m.s;
-          t.e[c] = m.e;
-        }
-      }
+      for (int b = threadIdx.x; b < ipp; b += blockDim.x) merge_part(t, &part[size_t(p) * bpp + b]);
       t = sq_warp_sum4(t);
       if (lane == 0) sh[warp] = t;   // warp 0 read sh before the barrier above
       __syncthreads();
       if (warp == 0) {
         const SqPart q = sq_block_tail(sh, lane, nw);
         if (lane == 0) {
-          psum[p] = sum4(sq_value(SqAcc{q.s[0], q.e[0]}), sq_value(SqAcc{q.s[1], q.e[1]}),
-                         sq_value(SqAcc{q.s[2], q.e[2]}), sq_value(SqAcc{q.s[3], q.e[3]}));
+          psum[p] = sum_of(q);
           cnt[p] = 0;
           __threadfence();
           flag[1] = (atomicAdd(ra.gcnt, 1) == nact - 1);
@@ -409,7 +440,7 @@ __device__ __forceinline__ void residual_items(const LevelDev& L, const Batch& B
       if (flag[1]) {   // every plane's sum is in: retire converged planes (App. B)
         __threadfence();
         retire_block(const_cast<int*>(B.act), const_cast<int*>(B.nact), psum, ra.S, ra.tol,
-                     ra.max_cycles, ra.stagnation, ra.use_cond, ra.handle, scan, ra.tail_planes);
+                     ra.max_cycles, ra.stagnation, ra.use_cond, ra.handle, scan, ra.tail_planes, RetireHint{});
         if (threadIdx.x == 0) *ra.gcnt = 0;
       }
     }
@@ -418,7 +449,7 @@ __device__ __forceinline__ void residual_items(const LevelDev& L, const Batch& B
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_residual(LevelDev L, Batch B, const double2* __restrict__ f,
+__global__ void __launch_bounds__(256, 5) k_residual(LevelDev L, Batch B, const double2* __restrict__ f,
                                                   const double2* __restrict__ u,
                                                   vec2_t<T>* __restrict__ r, SqPart* part,
                                                   Sum4* psum, int* cnt, int bpp, RetireArgs ra,
@@ -436,17 +467,27 @@ __global__ void __launch_bounds__(256) k_residual(LevelDev L, Batch B, const dou
   // Work items of CPT x 256 cells: with many planes active the per-item
   // reduction, fence and arrival count are paid once per 1024 cells; with few
   // planes every item is 256 cells, spreading a plane's FP64 work over more
-  // SMs.  bpp (the caller's) is the item count for CPT = 1.
+  // SMs.  bpp (the caller's) is the item count for CPT = 1.  Up to kFlatItems
+  // such items one arrival counter serves all planes and the last block sums every
+  // plane's items (a warp per plane) and retires: a round of fence, atomic and
+  // reload less (one plane of 128 x 64 cells: 7.9 us, 9.8 before; with up to
+  // 4096 items 10 planes of 256 x 128 took 24.5 us, 20.3 with a counter per
+  // plane: arrivals at one address queue).  48 registers (5 blocks an SM): with
+  // 56 the full batch of 256 x 128 took 111 us, 104 so.
+  const bool flat = nact * bpp <= kFlatItems && nact <= int(blockDim.x);
+  auto items = [&](auto zero, auto cpt, auto fl) {
+    residual_items<T, decltype(zero)::value, decltype(cpt)::value, decltype(fl)::value>(
+        L, B, f, u, r, part, psum, cnt, bpp, ra, ctab, dtab, nact, want_f, sh, flag, scan);
+  };
+  using one = std::integral_constant<int, 1>;
+  using four = std::integral_constant<int, 4>;
   if (r_is_f) {
-    if (nact >= 16)
-      residual_items<T, true, 4>(L, B, f, u, r, part, psum, cnt, bpp, ra, ctab, dtab, nact, want_f, sh, flag, scan);
-    else
-      residual_items<T, true, 1>(L, B, f, u, r, part, psum, cnt, bpp, ra, ctab, dtab, nact, want_f, sh, flag, scan);
+    if (nact >= 16) items(std::true_type{}, four{}, std::false_type{});
+    else items(std::true_type{}, one{}, std::false_type{});
   } else {
-    if (nact >= 16)
-      residual_items<T, false, 4>(L, B, f, u, r, part, psum, cnt, bpp, ra, ctab, dtab, nact, want_f, sh, flag, scan);
-    else
-      residual_items<T, false, 1>(L, B, f, u, r, part, psum, cnt, bpp, ra, ctab, dtab, nact, want_f, sh, flag, scan);
+    if (nact >= 16) items(std::false_type{}, four{}, std::false_type{});
+    else if (flat) items(std::false_type{}, one{}, std::true_type{});
+    else items(std::false_type{}, one{}, std::false_type{});
   }
 }
 
@@ -465,11 +506,11 @@ void launch_residual(const LevelDev& L, const Batch& B, const double2* f, const 
 
 __device__ void retire_block(int* act, int* nact, const Sum4* __restrict__ psum, RetireState S,
                              double tol, int max_cycles, int stagnation, int use_cond,
-                             unsigned long long handle, int* scan, int tail_planes) {
+                             unsigned long long handle, int* scan, int tail_planes, const RetireHint& hint) {
   __shared__ double smax[32];
   __shared__ int base_out;
-  const int n = *nact;
-  const int iter = *S.iter;
+  const int n = hint.n ? hint.n : *nact;
+  const int iter = hint.n ? hint.iter : *S.iter;
   const int tid = threadIdx.x;
   if (iter == 0) {
     double mx = 0.0;
@@ -489,7 +530,7 @@ __device__ void retire_block(int* act, int* nact, const Sum4* __restrict__ psum,
     }
     __syncthreads();
   }
-  const double floor2 = 1e-28 * (*S.fmax2);
+  const double floor2 = 1e-28 * (hint.n ? hint.fmax2 : *S.fmax2);
   const double tol2 = tol * tol;
   if (tid == 0) base_out = 0;
   __syncthreads();
@@ -497,10 +538,10 @@ __device__ void retire_block(int* act, int* nact, const Sum4* __restrict__ psum,
     const int k = c0 + tid;
     int keep = 0, p = -1;
     if (k < n) {
-      p = act[k];
+      p = hint.n ? hint.p : act[k];
       const Sum4 s = psum[p];
-      const double2 nf = S.nf2[p];
-      const double2 prev = S.nr2[p];
+      const double2 nf = hint.n ? hint.nf : S.nf2[p];
+      const double2 prev = hint.n ? hint.prev : S.nr2[p];
       const double tre = tol2 * fmax(nf.x, floor2), tim = tol2 * fmax(nf.y, floor2);
       int st = ST_ACTIVE;
       if (!isfinite(s.x) || !isfinite(s.y)) st = ST_NONFINITE;

@@ -152,3 +152,40 @@ def test_fused_first_level_held_in_registers(ps, nr, nt, large, nu1, nu2, n_sor,
         ref = u[1:-1, 1:-1].T
         assert np.abs(got[m].cpu().numpy() - ref).max() <= 1e-4 * np.abs(ref).max()
     s.close()
+
+
+# n_r, n_tz, n_phi: work items of 256 cells per launch of the residual, and its
+# arrivals: 3 (one per plane), 10, 160 (one counter for all), 288 and 384 (a
+# counter per plane until planes retire), and 16 planes and more
+RETIRE_GRIDS = [(8, 8, 4), (16, 32, 8), (128, 64, 8), (128, 64, 16), (256, 128, 4), (32, 32, 64)]
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("nr,nt,n_phi", RETIRE_GRIDS)
+def test_planes_retire_by_either_arrival_count(ps, nr, nt, n_phi, precision):
+    """A plane of zeros retires at once, every other one at the direct solution
+    (1e-9 at a relative residual of 1e-11), and a plane that is not finite
+    is reported without touching the others."""
+    import scipy.sparse.linalg as spla
+
+    from oracle import operator
+    sp = workloads.spec(workloads.SPHERICAL, nr, nt, n_phi, workloads.LOG, 1.0, 8.0)
+    s = ps.Solver.from_spec(sp, precision=precision, use_graph=False)
+    f = _planes((s.n_modes, nt, nr), nr + nt + n_phi)
+    f[1] = 0.0
+    u, cyc, rc = s.stage_mg_solve(torch.from_numpy(f).cuda(), tol=1e-11)
+    assert rc == ps.OK and cyc[1] == 0 and min(cyc[0], cyc[-1]) > 0
+    u = u.cpu().numpy()
+    assert not u[1].any()
+    p = oracle_plane(sp)
+    for m in (0, s.n_modes - 1):
+        A = operator.matrix(p, m).tocsc()
+        b = f[m].T
+        x = spla.spsolve(A, operator.to_vec(b.real)) + 1j * spla.spsolve(A, operator.to_vec(b.imag))
+        ref = operator.from_vec(x, nr, nt).T
+        assert np.abs(u[m] - ref).max() <= 1e-9 * np.abs(ref).max()
+    f[1] = np.nan
+    v, cyc2, rc = s.stage_mg_solve(torch.from_numpy(f).cuda(), tol=1e-11)
+    assert rc == ps.ERR_NONFINITE
+    assert cyc2[0] == cyc[0] and np.array_equal(v[0].cpu().numpy(), u[0])
+    s.close()
