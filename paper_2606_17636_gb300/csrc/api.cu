@@ -582,7 +582,16 @@ static int add_while(psolve_t h, cudaGraph_t graph, double tol, cudaStream_t bod
   if (cudaStreamBeginCaptureToGraph(body_st, body, nullptr, nullptr, 0,
                                     cudaStreamCaptureModeRelaxed) != cudaSuccess)
     return -1;
-  h->mg.loop_body(h->f, h->u, tol, body_st, 1, cond, few);
+  // Several iterations per pass of the WHILE node: a pass costs about 5 us of
+  // its own, an iteration that finds no active plane some 1.3 us a launch, and
+  // half the surplus is spent on average.  Bodies of few launches take 3 (128 x 64
+  // x 128 sphere: 984 us with 1, 948 with 2, 927 with 3, 930 with 4), those
+  // with one level-wide level 2 (FP64 cylinder of 32 x 32: 2524, 2488, 2464, 2458), longer
+  // ones 1 (FP64 sphere of 128 x 64: 7784 with 1, 7789 with 2).  The tail kernel
+  // takes its planes in the iteration that hands them over: 1.
+  const int base = h->mg.base;
+  const int passes = h->mg.tail_planes > 0 ? 1 : (few || base == 0 ? 3 : (base == 1 ? 2 : 1));
+  for (int k = 0; k < passes; ++k) h->mg.loop_body(h->f, h->u, tol, body_st, 1, cond, few);
   cudaGraph_t out;
   return cudaStreamEndCapture(body_st, &out) == cudaSuccess ? 0 : -1;
 }
