@@ -416,7 +416,7 @@ extern "C" void psolve_destroy(psolve_t h) {
   for (cudaEvent_t e : h->mark)
     if (e) cudaEventDestroy(e);
   if (h->gexec) cudaGraphExecDestroy(h->gexec);
-  if (h->mg.h_cont) cudaFreeHost(h->mg.h_cont);
+  h->mg.release_host();
   if (h->h_worst) cudaFreeHost(h->h_worst);
   h->A.release_all();
   delete h;

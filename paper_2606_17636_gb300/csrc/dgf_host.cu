@@ -157,7 +157,7 @@ static bool build_extended(const PlaneGeo& g, const Law& rlaw, const Law& tlaw,
     launch_ext_extract(ea, u, gt, int(p0), np, st);
   }
   cudaStreamSynchronize(st);
-  if (mg.h_cont) cudaFreeHost(mg.h_cont);
+  mg.release_host();
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { err = std::string("extended-domain DGF: ") + cudaGetErrorString(e); return false; }
   return true;

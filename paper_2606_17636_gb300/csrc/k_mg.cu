@@ -262,7 +262,7 @@ struct RetireHint {
 };
 __device__ void retire_block(int* act, int* nact, const Sum4* __restrict__ psum, RetireState S,
                              double tol, int max_cycles, int stagnation, int use_cond,
-                             unsigned long long handle, int* scan, int tail_planes, const RetireHint& hint);
+                             unsigned long long handle, int* scan, int tail_planes, int* host, const RetireHint& hint);
 
 // FP64 defect at (i, j) from the per-cell products (one FP64 operation for
 // the mode's diagonal read from its own table dm, five fused multiply-adds per
@@ -418,7 +418,7 @@ __device__ __forceinline__ void residual_items(const LevelDev& L, const Batch& B
       }
       __syncthreads();
       retire_block(const_cast<int*>(B.act), const_cast<int*>(B.nact), psum, ra.S, ra.tol, ra.max_cycles, ra.stagnation,
-                   ra.use_cond, ra.handle, scan, ra.tail_planes, hint);
+                   ra.use_cond, ra.handle, scan, ra.tail_planes, ra.host, hint);
       if (threadIdx.x == 0) *ra.gcnt = 0;
     } else if (flag[0]) {   // the plane's last item: its sums over the items in item order
       __threadfence();
@@ -440,7 +440,7 @@ __device__ __forceinline__ void residual_items(const LevelDev& L, const Batch& B
       if (flag[1]) {   // every plane's sum is in: retire converged planes (App. B)
         __threadfence();
         retire_block(const_cast<int*>(B.act), const_cast<int*>(B.nact), psum, ra.S, ra.tol,
-                     ra.max_cycles, ra.stagnation, ra.use_cond, ra.handle, scan, ra.tail_planes, RetireHint{});
+                     ra.max_cycles, ra.stagnation, ra.use_cond, ra.handle, scan, ra.tail_planes, ra.host, RetireHint{});
         if (threadIdx.x == 0) *ra.gcnt = 0;
       }
     }
@@ -506,7 +506,7 @@ void launch_residual(const LevelDev& L, const Batch& B, const double2* f, const 
 
 __device__ void retire_block(int* act, int* nact, const Sum4* __restrict__ psum, RetireState S,
                              double tol, int max_cycles, int stagnation, int use_cond,
-                             unsigned long long handle, int* scan, int tail_planes, const RetireHint& hint) {
+                             unsigned long long handle, int* scan, int tail_planes, int* host, const RetireHint& hint) {
   __shared__ double smax[32];
   __shared__ int base_out;
   const int n = hint.n ? hint.n : *nact;
@@ -581,6 +581,7 @@ __device__ void retire_block(int* act, int* nact, const Sum4* __restrict__ psum,
     *nact = base_out;
     *S.iter = iter + 1;
     *S.cont = cont;
+    if (host) *host = cont;
     if (use_cond) cudaGraphSetConditional(handle, cont == 1 ? 1u : 0u);
   }
 }

@@ -342,6 +342,7 @@ struct RetireArgs {
   int* gcnt;                   // completion counter, zero between launches
   int zero_guess;              // u is zero on the first iteration: r = f there
   int tail_planes;             // hand over to the tail kernel once at most this many remain (0: never)
+  int* host = nullptr;         // the continue flag's copy in pinned host memory (null: none)
 };
 
 // r = f - L u (FP64), stored as T2, and the volume-weighted norms per plane

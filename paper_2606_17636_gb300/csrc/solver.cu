@@ -361,7 +361,9 @@ bool MGSolver::init(Arena& A, const PlaneGeo& fine, bool neumann, const std::vec
   if (!d_fmax2 || !d_cnt || !d_gcnt) { err = "out of device memory"; return false; }
   cudaMemset(d_cnt, 0, sizeof(int) * mp);
   cudaMemset(d_gcnt, 0, sizeof(int));
-  if (cudaMallocHost(&h_cont, sizeof(int)) != cudaSuccess) { err = "pinned allocation failed"; return false; }
+  if (cudaMallocHost(&h_cont, kFlags * sizeof(int)) != cudaSuccess) { err = "pinned allocation failed"; return false; }
+  for (cudaEvent_t& ev : flag_at)
+    if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) { err = "event creation failed"; return false; }
   batch.act = d_act;
   batch.nact = d_nact;
   batch.slot = d_slot;
@@ -471,7 +473,7 @@ void MGSolver::fused(int lo, const VSmemArgs& v, cudaStream_t st) {
     launch_vsmem<double>(v, batch, (const double2*)f[lo], (double2*)e[lo], st);
 }
 void MGSolver::residual(const double2* ff, const double2* u, double tol, cudaStream_t st,
-                        int use_cond, unsigned long long cond, int hand_over) {
+                        int use_cond, unsigned long long cond, int hand_over, int* host) {
   RetireArgs ra;
   ra.S = S;
   ra.tol = tol;
@@ -482,6 +484,7 @@ void MGSolver::residual(const double2* ff, const double2* u, double tol, cudaStr
   ra.gcnt = d_gcnt;
   ra.zero_guess = zero_guess;
   ra.tail_planes = hand_over;
+  ra.host = host;
   if (opt.precision)
     launch_residual<float>(lv[0], batch, ff, u, (float2*)f[0], d_part, d_psum, d_cnt, ra, st, d_ctab, d_dtab);
   else
@@ -670,35 +673,58 @@ void MGSolver::loop_body(const double2* ff, double2* u, double tol, cudaStream_t
     launch_update<double>(lv[0], batch, u, (const double2*)e[0], st);
 }
 
+// The loop without a graph.  The host reads an iteration's continue flag while
+// the next iteration runs, which is enqueued before: once every plane has
+// retired the kernels find none active and change nothing.  The residual's
+// last block writes the flag to pinned memory itself, and an event behind that kernel
+// makes it visible: a copy in the stream stood between two kernels.  The tail
+// kernel takes its planes in the very iteration that hands them over, so with
+// a tail the flag is read at once.
 int MGSolver::eager_solve(const double2* ff, double2* u, double tol, cudaStream_t st,
                           std::string& err) {
   init_loop(st);
-  for (int phase = many_phase() ? 0 : 1; phase < (few_phase() ? 2 : 1); ++phase) {
-    bool handed = false;
-    for (int it = 0; it <= opt.max_cycles + 1 && !handed; ++it) {
-      residual(ff, u, tol, st, 0, 0, phase == 1 || !few_phase() ? tail_planes : few_planes);
-      cudaMemcpyAsync(h_cont, d_cont, sizeof(int), cudaMemcpyDeviceToHost, st);
-      const cudaError_t le = cudaGetLastError();
-      const cudaError_t se = cudaStreamSynchronize(st);
-      if (le != cudaSuccess || se != cudaSuccess) {
-        err = std::string("multigrid iteration: ") + cudaGetErrorString(le != cudaSuccess ? le : se);
-        return -2;
-      }
-      if (!*h_cont) return 0;
-      if (phase == 1) {
-        vcycle_few(st, u);
-      } else if (!vcycle(st, u)) {
-        if (opt.precision)
-          launch_update<float>(lv[0], batch, u, (const float2*)e[0], st);
-        else
-          launch_update<double>(lv[0], batch, u, (const double2*)e[0], st);
-      }
-      handed = *h_cont == 2;   // few planes remain: the next phase, or the tail kernel, takes them
+  const int lag = tail_planes > 0 ? 0 : 1;
+  static_assert(kFlags >= 2, "one flag is read while another is written");
+  bool few = !many_phase();
+  for (int it = 0; it <= opt.max_cycles + 1 + lag; ++it) {
+    residual(ff, u, tol, st, 0, 0, few || !few_phase() ? tail_planes : few_planes, h_cont + it % kFlags);
+    cudaEventRecord(flag_at[it % kFlags], st);
+    if (few) {
+      vcycle_few(st, u);
+    } else if (!vcycle(st, u)) {
+      if (opt.precision)
+        launch_update<float>(lv[0], batch, u, (const float2*)e[0], st);
+      else
+        launch_update<double>(lv[0], batch, u, (const double2*)e[0], st);
     }
-    if (!handed) return 0;
+    const int at = (it + kFlags - lag) % kFlags;
+    const cudaError_t le = cudaGetLastError();
+    const cudaError_t se = it >= lag ? cudaEventSynchronize(flag_at[at]) : cudaSuccess;
+    if (le != cudaSuccess || se != cudaSuccess) {
+      err = std::string("multigrid iteration: ") + cudaGetErrorString(le != cudaSuccess ? le : se);
+      return -2;
+    }
+    if (it < lag) continue;
+    if (!h_cont[at]) return 0;
+    if (h_cont[at] == 2) {   // few planes remain: the next phase, or the tail kernel, takes them
+      if (!few && few_phase()) {
+        few = true;
+      } else if (tail_planes > 0) {
+        tail(ff, u, tol, st);
+        return 0;
+      }
+    }
   }
-  tail(ff, u, tol, st);
   return 0;
+}
+
+void MGSolver::release_host() {
+  if (h_cont) cudaFreeHost(h_cont);
+  h_cont = nullptr;
+  for (cudaEvent_t& ev : flag_at) {
+    if (ev) cudaEventDestroy(ev);
+    ev = nullptr;
+  }
 }
 
 // A V-cycle of the last few planes: the window passes above level base.

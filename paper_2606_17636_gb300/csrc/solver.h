@@ -75,7 +75,12 @@ class MGSolver {
   double2* d_nr2 = nullptr;
   int* d_iter = nullptr;
   int* d_cont = nullptr;
-  int* h_cont = nullptr;   // pinned
+  // continue flags of the eager loop's iterations in flight (pinned, written by
+  // the residual) and the events behind those residuals
+  static constexpr int kFlags = 2;
+  int* h_cont = nullptr;
+  cudaEvent_t flag_at[kFlags] = {};
+  void release_host();
   Hierarchy H;
   std::vector<LevelDev> lv;
   Batch batch{};
@@ -110,7 +115,7 @@ class MGSolver {
   bool build_vsmem(Arena& A, int lo, int n_modes, VSmemArgs& v, std::string& err);
   // hand_over: the continue flag becomes 2 once at most that many planes remain
   void residual(const double2* f, const double2* u, double tol, cudaStream_t st, int use_cond,
-                unsigned long long cond, int hand_over);
+                unsigned long long cond, int hand_over, int* host = nullptr);
   // the defect alone into r (tolerance 0: no plane retires)
   void residual_to(const double2* f, const double2* u, void* r, cudaStream_t st);
   int* d_act = nullptr;
