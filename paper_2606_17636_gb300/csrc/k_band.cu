@@ -384,16 +384,6 @@ __global__ void __launch_bounds__(kBandThreads, 3)
   }
 }
 
-int band_sms() {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 132;
-  }
-  return sms;
-}
-
 bool run_length(int n) { return n >= 32 && n <= 512; }
 
 template <int CPL>
@@ -407,7 +397,7 @@ void radial(const LevelDev& L, const Batch& B, const float2* ein, float2* eout, 
     cudaFuncSetAttribute(k_band<CPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * kStages * 32 * CPL * 32);
     attr = true;
   }
-  const int resident = band_sms() * kBlocks * (kBandThreads / 32) * gpw;   // groups at once
+  const int resident = sm_count() * kBlocks * (kBandThreads / 32) * gpw;   // groups at once
   const long most = long(B.max_planes) * pairs;                            // bands of one pair
   const long warps = ((most < resident ? most : resident) + gpw - 1) / gpw;
   k_band<CPL><<<unsigned((warps + kBandThreads / 32 - 1) / (kBandThreads / 32)), kBandThreads, sm, st>>>(
@@ -418,7 +408,7 @@ template <int NS, bool UPD>
 void march(const LevelDev& L, const Batch& B, const float2* ein, float2* eout, const float2* f, double2* u,
            cudaStream_t st) {
   const int pairs = L.nr / 2, tiles = (pairs + 29) / 30, width = (pairs + tiles - 1) / tiles;
-  const int resident = band_sms() * 3 * (kBandThreads / 32);
+  const int resident = sm_count() * 3 * (kBandThreads / 32);
   const long most = long(B.max_planes) * tiles * (L.nt / 8);
   const long warps = most < resident ? most : resident;
   const size_t sm = (size_t(L.nt) + 8 * NS + (kBandThreads / 32) * kAhead * (UPD ? 8 : 4) * 32) * sizeof(float4);

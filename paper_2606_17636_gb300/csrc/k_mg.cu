@@ -47,7 +47,7 @@ enum { ST_ACTIVE = 1, ST_OK = 0, ST_STAGNATED = 2, ST_NOTCONV = -4, ST_NONFINITE
 // Grids of the per-plane kernels are bounded (a few blocks per SM) and loop
 // over work items w = k * bpp + b (active plane k, block b of bpp), so the
 // cost of a launch follows the active planes, not the planes allocated.
-static int work_grid(long items) {
+int sm_count() {
   static int sms = 0;   // cached on first use (the solver's set-up, before any capture)
   if (!sms) {
     int dev = 0;
@@ -55,9 +55,17 @@ static int work_grid(long items) {
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
       sms = 132;
   }
-  const long cap = long(sms) * 8;
+  return sms;
+}
+static int work_grid(long items) {
+  const long cap = long(sm_count()) * 8;
   return int(items < cap ? (items > 0 ? items : 1) : cap);
 }
+// Threads of a transfer's block: FP64 transfers are bound by the SM's FP64
+// units, so few cells are spread over more SMs (one plane of 128 x 64 cells:
+// 7.3 us with 8 blocks of 256, 5.0 with 32 of 64; 65 planes 22.8 either way).
+template <typename T>
+static int transfer_threads() { return sizeof(T) == 8 ? 64 : 256; }
 
 __device__ __forceinline__ bool plane_of(const Batch& B, int k, int& p, int& slot) {
   if (k >= *B.nact) return false;
@@ -139,7 +147,8 @@ template <typename T>
 void launch_restrict(const LevelDev& F, const LevelDev& C, const Batch& B, const vec2_t<T>* e,
                      const vec2_t<T>* f, vec2_t<T>* fc, cudaStream_t st) {
   const int n = C.nr * C.nt;
-  k_restrict<T><<<work_grid(long((n + 255) / 256) * B.max_planes), 256, 0, st>>>(F, C, B, e, f, fc);
+  const int th = transfer_threads<T>();
+  k_restrict<T><<<work_grid(long((n + th - 1) / th) * B.max_planes), th, 0, st>>>(F, C, B, e, f, fc);
 }
 
 // ---------------------------------------------------------------------------
@@ -219,7 +228,8 @@ template <typename T>
 void launch_prolong(const LevelDev& F, const LevelDev& C, const Batch& B, vec2_t<T>* e,
                     const vec2_t<T>* ec, cudaStream_t st) {
   const int n = C.nr * C.nt;
-  k_prolong<T><<<work_grid(long((n + 255) / 256) * B.max_planes), 256, 0, st>>>(F, C, B, e, ec);
+  const int th = transfer_threads<T>();
+  k_prolong<T><<<work_grid(long((n + th - 1) / th) * B.max_planes), th, 0, st>>>(F, C, B, e, ec);
 }
 
 // ---------------------------------------------------------------------------
@@ -336,6 +346,9 @@ __device__ __forceinline__ Sum4 sum_of(const SqPart& q) {
 }
 
 constexpr int kFlatItems = 256;
+// Blocks that 1024-cell items must give (two an SM); with fewer, 256-cell items
+// use more SMs (17 planes of 32 x 32 cells, FP64: 8.2 us, 14.2 with 17 blocks).
+constexpr int kWideBlocks = 304;
 
 // The residual work items of one launch.  ZERO: u = 0 on the first
 // iteration, so r = f and |r|^2 = |f|^2 (no stencil); CPT: cells per thread
@@ -464,9 +477,9 @@ __global__ void __launch_bounds__(256, 5) k_residual(LevelDev L, Batch B, const 
   const bool want_f = *ra.S.iter == 0;     // |f| is needed on the first iteration only
   // from a zero initial guess the first defect is f itself (no stencil)
   const bool r_is_f = want_f && ra.zero_guess;
-  // Work items of CPT x 256 cells: with many planes active the per-item
+  // Work items of CPT x 256 cells: with many cells active the per-item
   // reduction, fence and arrival count are paid once per 1024 cells; with few
-  // planes every item is 256 cells, spreading a plane's FP64 work over more
+  // cells every item is 256 cells, spreading a plane's FP64 work over more
   // SMs.  bpp (the caller's) is the item count for CPT = 1.  Up to kFlatItems
   // such items one arrival counter serves all planes and the last block sums every
   // plane's items (a warp per plane) and retires: a round of fence, atomic and
@@ -481,11 +494,12 @@ __global__ void __launch_bounds__(256, 5) k_residual(LevelDev L, Batch B, const 
   };
   using one = std::integral_constant<int, 1>;
   using four = std::integral_constant<int, 4>;
+  const bool wide = nact >= 16 && nact * bpp >= 4 * kWideBlocks;
   if (r_is_f) {
-    if (nact >= 16) items(std::true_type{}, four{}, std::false_type{});
+    if (wide) items(std::true_type{}, four{}, std::false_type{});
     else items(std::true_type{}, one{}, std::false_type{});
   } else {
-    if (nact >= 16) items(std::false_type{}, four{}, std::false_type{});
+    if (wide) items(std::false_type{}, four{}, std::false_type{});
     else if (flat) items(std::false_type{}, one{}, std::true_type{});
     else items(std::false_type{}, one{}, std::false_type{});
   }

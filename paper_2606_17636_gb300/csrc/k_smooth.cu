@@ -22,13 +22,24 @@
 
 namespace ps {
 
-// Blocks per plane for the active count: base * mult, mult in {1, 2, 4},
-// mult <= cap.
+// Blocks per plane for the active count: base * mult, mult in {1, 2, 4}
+// (FP64: to 16), mult <= cap.
+template <typename T>
 __device__ __forceinline__ int spread(int base, int nact, int cap) {
   const int G = int(gridDim.x * gridDim.y);
   int mult = 1;
-  while (mult < 4 && mult < cap && nact * base * mult * 2 <= G) mult *= 2;
+  while (mult < (sizeof(T) == 8 ? 16 : 4) && mult < cap && nact * base * mult * 2 <= G) mult *= 2;
   return mult;
+}
+// Rows of the grid: a plane each; FP64 passes, bound by an SM's FP64 units,
+// have at least a block per SM, so that narrower tiles spread few or small
+// planes over all of them (17 planes of 32 x 32 cells had 17 SMs at work on a
+// polar pass, 15.7 us; with 136 blocks of 4 columns 6.5).
+template <typename T>
+static int grid_rows(int base, int planes) {
+  if (sizeof(T) == 4) return planes;
+  const int fill = (sm_count() + base - 1) / base;
+  return planes > fill ? planes : fill;
 }
 
 
@@ -61,7 +72,7 @@ __global__ void __launch_bounds__(256) k_rpass2(LevelDev L, Batch B, const vec2_
   typedef vec2_t<T> V;
   extern __shared__ __align__(16) unsigned char sraw[];
   const int nact = *B.nact;
-  const int mult = spread(int(gridDim.x), nact, Wmax / 2);
+  const int mult = spread<T>(int(gridDim.x), nact, Wmax / 2);
   const int per = int(gridDim.x) * mult;
   const int b = int(blockIdx.y * gridDim.x + blockIdx.x);
   const int k = b / per;
@@ -145,7 +156,7 @@ __global__ void __launch_bounds__(256) k_tpass2(LevelDev L, Batch B, const vec2_
   typedef vec2_t<T> V;
   extern __shared__ __align__(16) unsigned char sraw[];
   const int nact = *B.nact;
-  const int mult = spread(int(gridDim.x), nact, TWmax / 2);
+  const int mult = spread<T>(int(gridDim.x), nact, TWmax / 2);
   const int per = int(gridDim.x) * mult;
   const int b = int(blockIdx.y * gridDim.x + blockIdx.x);
   const int kp = b / per;
@@ -252,7 +263,8 @@ static void rpass2(const LevelDev& L, const Batch& B, const vec2_t<T>* ein, vec2
     cudaFuncSetAttribute(k_rpass2<T, CPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     attr = true;
   }
-  dim3 grid((L.nt + Wmax - 1) / Wmax, B.max_planes);
+  const int per = (L.nt + Wmax - 1) / Wmax;
+  dim3 grid(per, grid_rows<T>(per, B.max_planes));
   k_rpass2<T, CPL><<<grid, 32 * Wmax, sm, st>>>(L, B, ein, eout, f, zi ? 1 : 0, n_sor, Wmax);
 }
 
@@ -266,7 +278,7 @@ static void tpass2(const LevelDev& L, const Batch& B, const vec2_t<T>* ein, vec2
     cudaFuncSetAttribute(k_tpass2<T, CPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     attr = true;
   }
-  dim3 grid(L.nr / TW, B.max_planes);
+  dim3 grid(L.nr / TW, grid_rows<T>(L.nr / TW, B.max_planes));
   k_tpass2<T, CPL><<<grid, 256, sm, st>>>(L, B, ein, eout, f, n_sor, TW, u);
 }
 

@@ -423,16 +423,6 @@ __global__ void __launch_bounds__(WX * WY / 16, 8192 / (WX * WY)) k_tile(LevelDe
 
 int tile_count(int n, int W, int H) { return n <= W ? 1 : (n - 2 * H + (W - 2 * H) - 1) / (W - 2 * H); }
 
-int sm_count() {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 132;
-  }
-  return sms;
-}
-
 int win(int n) { return n >= 64 ? 64 : 32; }
 
 template <int WX, int WY>

@@ -245,6 +245,8 @@ void launch_smooth(const LevelDev& L, const Batch& B, vec2_t<T>* e, const vec2_t
                    vec2_t<T>* tmp, int cycles, int n_sor, bool zero_init, Tiles tiles,
                    cudaStream_t st, double2* u = nullptr);
 
+// SMs of the current device (queried once, in a solver's set-up before any capture).
+int sm_count();
 // The same passes for FP32 lines of 32 to 512 cells held in registers
 // (k_band.cu: radial bands, polar marches), where they pay.
 bool band_pays(int nr, int nt, int n_sor, int planes);
