@@ -43,6 +43,13 @@ static int grid_rows(int base, int planes) {
 }
 
 
+// FP64 lines of up to 256 cells read their inverse diagonals (longer ones have
+// no registers left for them).  65 planes of 128 x 64 cells, radial / polar
+// pass: 32.8 / 33.9 us, 40.7 / 40.8 with the diagonal formed in the pass; one
+// plane 9.8 / 7.2, 11.8 / 8.0.
+template <typename T, int CPL>
+constexpr bool kIds = sizeof(T) == 8 && CPL <= 8;
+
 // Radial pass, both colours: a block of 32 Wmax threads owns W lines
 // [j0, j0+W), W = Wmax / mult.
 // Every line it reads is first staged in shared memory with asynchronous
@@ -89,6 +96,19 @@ __global__ void __launch_bounds__(256) k_rpass2(LevelDev L, Batch B, const vec2_
   const size_t base = size_t(p) * nr * nt;
   stage_lines<T>(se, ein + base, j0 - 1, W + 3, nr, nt, zero_init != 0);
   stage_lines<T>(sf, f + base, j0, W + 1, nr, nt, false);
+  // FP64: this warp's two lines' inverse diagonals, loaded meanwhile (the FP64
+  // units bound the pass; a reciprocal and its operands are a third of a
+  // line's operations)
+  double id0[CPL], id1[CPL];
+  bool pre = false;
+  if constexpr (kIds<T, CPL>) {
+    pre = L.idr != nullptr;
+    if (pre) {
+      const double* t = L.idr + size_t(slot) * nr * nt;
+      if (warp <= W / 2) ld_ids<CPL>(id0, t + size_t(min(j0 + 2 * warp, nt - 1)) * nr, lane, nr);
+      if (warp < W / 2) ld_ids<CPL>(id1, t + size_t(min(j0 + 1 + 2 * warp, nt - 1)) * nr, lane, nr);
+    }
+  }
   cp_async_wait_all();
   __syncthreads();
   const T* rt = rt_<T>(L);
@@ -104,7 +124,12 @@ __global__ void __launch_bounds__(256) k_rpass2(LevelDev L, Batch B, const vec2_
       ld_line<V, CPL>(un, eline(j + 1), lane, nr);
       ld_line<V, CPL>(us, eline(j - 1), lane, nr);
       ld_line<V, CPL>(g, sf + size_t(j - j0) * nr, lane, nr);
-      relax_r<T, CPL>(L, rt, tt, s2, om[j], j, g, un, us, n_sor, ev);
+      if constexpr (kIds<T, CPL>) {
+        if (pre) relax_r<T, CPL, true>(L, rt, tt, s2, om[j], j, g, un, us, n_sor, ev, id0);
+        else relax_r<T, CPL>(L, rt, tt, s2, om[j], j, g, un, us, n_sor, ev);
+      } else {
+        relax_r<T, CPL>(L, rt, tt, s2, om[j], j, g, un, us, n_sor, ev);
+      }
       st_line<V, CPL>(s0 + warp * nr, ev, lane, nr);
     }
   }
@@ -122,7 +147,12 @@ __global__ void __launch_bounds__(256) k_rpass2(LevelDev L, Batch B, const vec2_
 #pragma unroll
         for (int c = 0; c < CPL; ++c) un[c] = z2<V>();
       }
-      relax_r<T, CPL>(L, rt, tt, s2, om[j], j, g, un, us, n_sor, ev);
+      if constexpr (kIds<T, CPL>) {
+        if (pre) relax_r<T, CPL, true>(L, rt, tt, s2, om[j], j, g, un, us, n_sor, ev, id1);
+        else relax_r<T, CPL>(L, rt, tt, s2, om[j], j, g, un, us, n_sor, ev);
+      } else {
+        relax_r<T, CPL>(L, rt, tt, s2, om[j], j, g, un, us, n_sor, ev);
+      }
       st_line<V, CPL>(eout + base + size_t(j) * nr, ev, lane, nr);
     }
   } else if (warp < W) {          // store the block's colour-0 lines
@@ -178,13 +208,24 @@ __global__ void __launch_bounds__(256) k_tpass2(LevelDev L, Batch B, const vec2_
     cp_async_v(se + o, ein + g, in);
     cp_async_v(sf + o, f + g, in);
   }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  // FP64: the inverse diagonals of this warp's first column, loaded meanwhile,
+  // then always the next column's while one is relaxed
+  double idn[CPL];
+  bool pre = false;
+  auto ids = [&](int i) {
+    if constexpr (kIds<T, CPL>) ld_ids<CPL>(idn, L.idt + (size_t(slot) * nr + (i < nr ? i : 0)) * nt, lane, nt);
+  };
+  if constexpr (kIds<T, CPL>) {
+    pre = L.idt != nullptr;
+    if (pre) ids(i0 + 2 * warp);
+  }
   cp_async_wait_all();
   __syncthreads();
   const T* rt = rt_<T>(L);
   const T* tt = tt_<T>(L);
   const T s2 = s2_<T>(B, slot);
   const T* om = omt_<T>(L) + size_t(slot) * nr;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const bool on = CPL > 1 || lane < nt;
   for (int color = 0; color < 2; ++color) {
     const int ncol = color == 0 ? TW / 2 + 1 : TW / 2;   // colour 0 includes column i0+TW
@@ -204,7 +245,20 @@ __global__ void __launch_bounds__(256) k_tpass2(LevelDev L, Batch B, const vec2_
           g[c] = sf[tslot<CPL>(j, cc, SW)];
         }
       }
-      relax_t<T, CPL>(L, rt, tt, s2, om[i], i, g, ue, uw, n_sor, ev);
+      if constexpr (kIds<T, CPL>) {
+        if (pre) {
+          double id[CPL];
+#pragma unroll
+          for (int c = 0; c < CPL; ++c) id[c] = idn[c];
+          if (k + nw < ncol && i + 2 * nw < nr) ids(i + 2 * nw);
+          else if (color == 0 && warp < TW / 2) ids(i0 + 1 + 2 * warp);
+          relax_t<T, CPL, true>(L, rt, tt, s2, om[i], i, g, ue, uw, n_sor, ev, id);
+        } else {
+          relax_t<T, CPL>(L, rt, tt, s2, om[i], i, g, ue, uw, n_sor, ev);
+        }
+      } else {
+        relax_t<T, CPL>(L, rt, tt, s2, om[i], i, g, ue, uw, n_sor, ev);
+      }
       if (on) {
 #pragma unroll
         for (int c = 0; c < CPL; ++c) se[tslot<CPL>(lcell<CPL>(lane, c), cc, SW)] = ev[c];
@@ -308,6 +362,25 @@ static void tpass2_any(const LevelDev& L, const Batch& B, const vec2_t<T>* ein, 
     case 32: tpass2<T, 32>(L, B, ein, eout, f, n_sor, cols, u, st); break;
     default: std::fprintf(stderr, "psolve: polar size %d unsupported\n", L.nt);
   }
+}
+
+__global__ void k_inverse_diagonal(LevelDev L, const double* __restrict__ s2d, int slots, double* __restrict__ idr,
+                                   double* __restrict__ idt) {
+  const int nr = L.nr, nt = L.nt, NR = nr + 2, NT = nt + 2;
+  const size_t n = size_t(nr) * nt;
+  for (size_t q = blockIdx.x * size_t(blockDim.x) + threadIdx.x; q < n * slots; q += size_t(gridDim.x) * blockDim.x) {
+    const size_t slot = q / n, c = q - slot * n;
+    const int j = int(c / nr), i = int(c - size_t(j) * nr);
+    const double d = fmac(-(s2d[slot] * L.rd[RT_Q * NR + i + 1]), L.td[TT_T * NT + j + 1],
+                          fmac(L.rd[RT_P * NR + i + 1], L.td[TT_DT * NT + j + 1], L.rd[RT_DR * NR + i + 1]));
+    const double v = rcp_diag(d);   // the passes' own value
+    idr[q] = v;
+    idt[(slot * nr + i) * nt + j] = v;
+  }
+}
+
+void launch_inverse_diagonal(const LevelDev& L, const double* s2d, int slots, double* idr, double* idt, cudaStream_t st) {
+  k_inverse_diagonal<<<8 * sm_count(), 256, 0, st>>>(L, s2d, slots, idr, idt);
 }
 
 template <typename T>

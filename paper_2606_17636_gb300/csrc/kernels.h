@@ -187,7 +187,13 @@ struct LevelDev {
   const float* omr_f;
   const float* omt_f;
   int gL, gR, gB, gT;   // coarse-ghost rules when this level is prolongated from
+  // FP64 inverse diagonals per slot, cells of a radial line or of a polar line
+  // contiguous ([slots][nt][nr], [slots][nr][nt]); null: formed in the passes
+  const double* idr = nullptr;
+  const double* idt = nullptr;
 };
+// Fills them (device pointers) from the level's tables.
+void launch_inverse_diagonal(const LevelDev& L, const double* s2d, int slots, double* idr, double* idt, cudaStream_t st);
 
 // A batch of planes: plane p of a level buffer starts at p * nr * nt; its
 // mode slot is slot[p] (identity when slot == nullptr); the mode's

@@ -295,12 +295,12 @@ __device__ __forceinline__ void relax_r(const LevelDev& L, const RLineTabs<T, CP
 
 // Same, loading the coefficients from the level's table as it uses them (for
 // kernels without registers to keep them): neighbour lines first (they die
-// there), then the diagonal, then the along-line couplings.
-template <typename T, int CPL>
+// there), then the diagonal (PRE: given, idp), then the along-line couplings.
+template <typename T, int CPL, bool PRE = false>
 __device__ __forceinline__ void relax_r(const LevelDev& L, const T* rt, const T* tt, T s2, T w,
                                         int j, vec2_t<T> (&g)[CPL], const vec2_t<T> (&un)[CPL],
                                         const vec2_t<T> (&us)[CPL], int n_sor,
-                                        vec2_t<T> (&ev)[CPL]) {
+                                        vec2_t<T> (&ev)[CPL], const T* idp = nullptr) {
   const int lane = threadIdx.x & 31, nr = L.nr, NR = nr + 2, NT = L.nt + 2;
   const T aN = tt[TT_AN * NT + j + 1], aS = tt[TT_AS * NT + j + 1];
   const T Tj = tt[TT_T * NT + j + 1], dtj = tt[TT_DT * NT + j + 1];
@@ -312,7 +312,10 @@ __device__ __forceinline__ void relax_r(const LevelDev& L, const T* rt, const T*
     g[c].x = fmac(-P[c], fmac(aS, us[c].x, aN * un[c].x), g[c].x);
     g[c].y = fmac(-P[c], fmac(aS, us[c].y, aN * un[c].y), g[c].y);
   }
-  {
+  if constexpr (PRE) {
+#pragma unroll
+    for (int c = 0; c < CPL; ++c) id[c] = idp[c];
+  } else {
     T dr[CPL], q[CPL];
     ld_tab<T, CPL>(dr, rt + RT_DR * NR, lane, nr);
     ld_tab<T, CPL>(q, rt + RT_Q * NR, lane, nr);
@@ -349,12 +352,12 @@ __device__ __forceinline__ void relax_t(const LevelDev& L, const T* rt, const TL
   sor_line<T, CPL>(ev, g, up, dn, id, w, nt, n_sor);
 }
 
-// Same, loading the coefficients as it uses them.
-template <typename T, int CPL>
+// Same, loading the coefficients as it uses them (PRE: the inverse diagonal is given).
+template <typename T, int CPL, bool PRE = false>
 __device__ __forceinline__ void relax_t(const LevelDev& L, const T* rt, const T* tt, T s2, T w,
                                         int i, vec2_t<T> (&g)[CPL], const vec2_t<T> (&ue)[CPL],
                                         const vec2_t<T> (&uw)[CPL], int n_sor,
-                                        vec2_t<T> (&ev)[CPL]) {
+                                        vec2_t<T> (&ev)[CPL], const T* idp = nullptr) {
   const int lane = threadIdx.x & 31, nt = L.nt, NR = L.nr + 2, NT = nt + 2;
   const T P = rt[RT_P * NR + i + 1], aE = rt[RT_AE * NR + i + 1], aW = rt[RT_AW * NR + i + 1];
   const T dr = rt[RT_DR * NR + i + 1], Qi = rt[RT_Q * NR + i + 1];
@@ -365,7 +368,10 @@ __device__ __forceinline__ void relax_t(const LevelDev& L, const T* rt, const T*
     g[c].x = fmac(-aW, uw[c].x, fmac(-aE, ue[c].x, g[c].x));
     g[c].y = fmac(-aW, uw[c].y, fmac(-aE, ue[c].y, g[c].y));
   }
-  {
+  if constexpr (PRE) {
+#pragma unroll
+    for (int c = 0; c < CPL; ++c) id[c] = idp[c];
+  } else {
     T dt[CPL], tj[CPL];
     ld_tab<T, CPL>(dt, tt + TT_DT * NT, lane, nt);
     ld_tab<T, CPL>(tj, tt + TT_T * NT, lane, nt);
@@ -380,6 +386,21 @@ __device__ __forceinline__ void relax_t(const LevelDev& L, const T* rt, const T*
     dn[c] = P * dn[c];
   }
   sor_line<T, CPL>(ev, g, up, dn, id, w, nt, n_sor);
+}
+
+// The lane's inverse diagonals of a line of n cells stored contiguously at p.
+template <int CPL>
+__device__ __forceinline__ void ld_ids(double (&d)[CPL], const double* p, int lane, int n) {
+  if constexpr (CPL == 1) {
+    d[0] = lane < n ? __ldg(p + lane) : 0.0;
+  } else {
+#pragma unroll
+    for (int q = 0; q < CPL / 2; ++q) {
+      const double2 v = __ldg(reinterpret_cast<const double2*>(p + 2 * lane + 64 * q));
+      d[2 * q] = v.x;
+      d[2 * q + 1] = v.y;
+    }
+  }
 }
 
 // ---- runs of consecutive cells per lane (FP32) ----------------------------------

@@ -334,6 +334,26 @@ bool MGSolver::init(Arena& A, const PlaneGeo& fine, bool neumann, const std::vec
     base = nl - 1;
     if (!build_vsmem(A, base, int(modes.size()), vsb, err)) return false;
   }
+  if (!opt.precision) {
+    // FP64 smoothing: inverse diagonals per mode and cell of the levels on the
+    // line passes, where they take at most an eighth of the free memory (the
+    // passes form them otherwise)
+    size_t need = 0, free_b = 0, total_b = 0;
+    for (int l = 0; l < base; ++l) need += 2 * sizeof(double) * modes.size() * size_t(lv[l].nr) * lv[l].nt;
+    if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && need <= free_b / 8) {
+      for (int l = 0; l < base; ++l) {
+        const size_t bytes = sizeof(double) * modes.size() * size_t(lv[l].nr) * lv[l].nt;
+        double* a = static_cast<double*>(A.get(bytes));
+        double* b = static_cast<double*>(A.get(bytes));
+        if (!a || !b) break;
+        launch_inverse_diagonal(lv[l], d_s2, int(modes.size()), a, b, 0);
+        lv[l].idr = a;
+        lv[l].idt = b;
+      }
+      cudaGetLastError();
+      if (cudaStreamSynchronize(0) != cudaSuccess) { err = "inverse diagonals"; return false; }
+    }
+  }
   if (opt.precision && base > 0) {   // the window passes' buffers; without them every plane stays with the level-wide passes
     tmp2 = A.get(size_t(mp) * lv[0].nr * lv[0].nt * vb);
     e2.assign(nl, nullptr);

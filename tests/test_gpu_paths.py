@@ -189,3 +189,33 @@ def test_planes_retire_by_either_arrival_count(ps, nr, nt, n_phi, precision):
     assert rc == ps.ERR_NONFINITE
     assert cyc2[0] == cyc[0] and np.array_equal(v[0].cpu().numpy(), u[0])
     s.close()
+
+
+# n_r, n_tz, n_phi: enough planes for whole tiles at first (a warp relaxes
+# several columns in turn), narrower ones as they retire; lines of one, two and
+# four cells a lane
+FP64_MANY = [(32, 32, 256), (64, 32, 128), (32, 64, 128), (128, 64, 128)]
+
+
+@pytest.mark.parametrize("nr,nt,n_phi", FP64_MANY)
+def test_fp64_solves_with_stored_inverse_diagonals(ps, nr, nt, n_phi):
+    """Many planes on the FP64 line passes: the direct solution to 1e-10 at a
+    relative residual of 1e-12, and the oracle's cycle counts."""
+    import scipy.sparse.linalg as spla
+
+    from oracle import mg, operator
+    sp = workloads.spec(workloads.SPHERICAL, nr, nt, n_phi, workloads.LOG, 1.0, 8.0)
+    s = ps.Solver.from_spec(sp, precision=ps.FP64, use_graph=False)
+    f = _planes((s.n_modes, nt, nr), nr + nt)
+    u, cyc, rc = s.stage_mg_solve(torch.from_numpy(f).cuda(), tol=1e-12)
+    assert rc == ps.OK
+    p = oracle_plane(sp)
+    H = mg.Hierarchy(p)
+    for m in (0, 1, s.n_modes - 1):
+        A = operator.matrix(p, m).tocsc()
+        b = f[m].T
+        x = spla.spsolve(A, operator.to_vec(b.real)) + 1j * spla.spsolve(A, operator.to_vec(b.imag))
+        ref = operator.from_vec(x, nr, nt).T
+        assert np.abs(u[m].cpu().numpy() - ref).max() <= 1e-10 * np.abs(ref).max()
+        assert abs(cyc[m] - H.solve(m, b, 1e-12)[1]) <= 1
+    s.close()
