@@ -592,7 +592,9 @@ def launches_per_solve(s, st):
     the loop runs I + 1 residuals and I V-cycles; with the cluster-resident
     tail (P planes) it hands over after the first iteration k that leaves at
     most P planes active (k + 1 residuals and V-cycles), then one tail
-    launch finishes them."""
+    launch finishes them.  A captured graph runs whole passes of several
+    iterations, the last ones with no plane active, and the mixed path's
+    last few planes take the window passes (psolve_get_loops)."""
     sc = s.schedule()
     first = s.fused_level()
     vcycle = first * (2 * sc["nu_pre"] + 1 + 1 + 2 * sc["nu_post"]) + 1   # + fused
@@ -600,7 +602,38 @@ def launches_per_solve(s, st):
     fixed = 1 + 1 + 3 + 1 + 1 + 1           # fft, init x2, screening/boundary/ghosts, ifft, status
     tail_planes = s.tail()[0]
 
+    shape = s.loops() if hasattr(s, "loops") else None
+
+    def phases(cycles):
+        """Graph loops without the tail: passes of the first loop until at most
+        few_planes remain, the hand-over kernel, passes of the second."""
+        n, it = 0, 0
+        left = lambda k: sum(1 for c in cycles if c > k)   # active after residual k
+        many = 2 - shape["fused_update"]
+        for lev in range(shape["level_wide"]):   # FP64: levels from `first` on with their own counts
+            own = lev >= first
+            a = own and sc["nu_pre_fused"] or sc["nu_pre"]
+            b = own and sc["nu_post_fused"] or sc["nu_post"]
+            many += 2 * a + 2 + 2 * b
+        few = shape["few_planes"]
+        if few < len(cycles):
+            go = True
+            while go:
+                n += shape["passes"] * (1 + many)
+                it += shape["passes"]
+                go = left(it - 1) > few
+        if few > 0:
+            n += 1 if few < len(cycles) else 0
+            go = it == 0 or left(it - 1) > 0
+            while go:
+                n += shape["few_passes"] * (1 + shape["few_launches"])
+                it += shape["few_passes"]
+                go = left(it - 1) > 0
+        return n
+
     def loop(cycles):
+        if shape is not None and tail_planes == 0:
+            return phases(cycles)
         it = max(cycles)
         if tail_planes > 0:
             for k in range(it):

@@ -276,6 +276,18 @@ int psolve_set_stream(psolve_t h, void* cuda_stream);
 int psolve_set_tail(psolve_t h, int max_planes);
 int psolve_get_tail(psolve_t h, int* planes, int* cluster_ctas);
 
+/* The launches of a handle's multigrid loops: level_wide = levels smoothed by
+ * level-wide passes (the fused V-cycle kernel takes the rest); few_planes =
+ * active planes from which on the mixed path's window passes take those levels
+ * (0: never), few_launches = launches of such a V-cycle; passes and few_passes
+ * = iterations per pass of the captured graph's loops before and after that;
+ * fused_update = 1 when the update is part of the V-cycle's last launch.
+ * PSOLVE_OK, or PSOLVE_ERR_ARG for a null argument. */
+typedef struct {
+  int level_wide, few_planes, few_launches, passes, few_passes, fused_update;
+} psolve_loops;
+int psolve_get_loops(psolve_t h, psolve_loops* out);
+
 /* Smoothing schedule and tile shapes of a handle.  Sec. 3.2 leaves the
  * schedule open (a small number of smoothing cycles per level, typically two
  * or three, and a few SOR sweeps per line); it changes the convergence rate,

@@ -46,6 +46,11 @@ class Stats(ctypes.Structure):
                 ("status", ctypes.POINTER(ctypes.c_int))]
 
 
+class Loops(ctypes.Structure):
+    _fields_ = [(k, ctypes.c_int) for k in ("level_wide", "few_planes", "few_launches", "passes", "few_passes",
+                                            "fused_update")]
+
+
 class Schedule(ctypes.Structure):
     _fields_ = [("nu_pre", ctypes.c_int), ("nu_post", ctypes.c_int), ("n_sor", ctypes.c_int),
                 ("lines_r", ctypes.c_int), ("cols_t", ctypes.c_int), ("nu_pre_fused", ctypes.c_int),
@@ -121,6 +126,7 @@ def lib():
             "psolve_set_warm_start": (I, [P, I]),
             "psolve_set_tail": (I, [P, I]),
             "psolve_get_tail": (I, [P, ctypes.POINTER(I), ctypes.POINTER(I)]),
+            "psolve_get_loops": (I, [P, ctypes.POINTER(Loops)]),
             "psolve_get_fused_level": (I, [P, ctypes.POINTER(ctypes.c_int)]),
             "psolve_stage_restrict": (I, [P, I, I, P, P, P]),
             "psolve_stage_residual": (I, [P, I, P, P, P]),
@@ -272,6 +278,12 @@ class Solver:
         p, c = ctypes.c_int(), ctypes.c_int()
         check(lib().psolve_get_tail(self.h, ctypes.byref(p), ctypes.byref(c)), "psolve_get_tail")
         return p.value, c.value
+
+    def loops(self):
+        """The launches of the multigrid loops (psolve_loops) as a dict."""
+        o = Loops()
+        check(lib().psolve_get_loops(self.h, ctypes.byref(o)), "psolve_get_loops")
+        return {k: getattr(o, k) for k, _ in Loops._fields_}
 
     def close(self):
         if getattr(self, "h", None):

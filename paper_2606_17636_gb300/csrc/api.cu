@@ -473,6 +473,21 @@ extern "C" int psolve_set_tail(psolve_t h, int max_planes) {
   return cuda_ok("set_tail") ? PSOLVE_OK : PSOLVE_ERR_CUDA;
 }
 
+static int loop_passes(psolve_t h, bool few);
+extern "C" int psolve_get_loops(psolve_t h, psolve_loops* out) {
+  if (!h || !out) return fail(PSOLVE_ERR_ARG, "null argument");
+  const MGSolver& m = h->mg;
+  out->level_wide = m.base;
+  out->few_planes = m.few_planes;
+  out->few_launches = 1;
+  for (const auto* legs : {&m.t_down, &m.t_up})
+    for (const auto& leg : *legs) out->few_launches += int(leg.size());
+  out->passes = loop_passes(h, false);
+  out->few_passes = loop_passes(h, true);
+  out->fused_update = m.base > 0 && m.opt.nu2 > 0 ? 1 : 0;
+  return PSOLVE_OK;
+}
+
 extern "C" int psolve_get_tail(psolve_t h, int* planes, int* cluster_ctas) {
   if (!h) return fail(PSOLVE_ERR_ARG, "null handle");
   if (planes) *planes = h->mg.tail_planes;
@@ -556,6 +571,18 @@ __global__ void k_hand_over(const int* cont, cudaGraphConditionalHandle cond) {
   cudaGraphSetConditional(cond, *cont == 2 ? 1u : 0u);
 }
 
+// Several iterations per pass of the WHILE node: a pass costs about 5 us of
+// its own, an iteration that finds no active plane some 1.3 us a launch, and
+// half the surplus is spent on average.  Bodies of few launches take 3 (128 x 64
+// x 128 sphere: 984 us with 1, 948 with 2, 927 with 3, 930 with 4), those
+// with one level-wide level 2 (FP64 cylinder of 32 x 32: 2524, 2488, 2464, 2458), longer
+// ones 1 (FP64 sphere of 128 x 64: 7784 with 1, 7789 with 2).  The tail kernel
+// takes its planes in the iteration that hands them over: 1.
+static int loop_passes(psolve_t h, bool few) {
+  const int base = h->mg.base;
+  return h->mg.tail_planes > 0 ? 1 : (few || base == 0 ? 3 : (base == 1 ? 2 : 1));
+}
+
 static int add_while(psolve_t h, cudaGraph_t graph, double tol, cudaStream_t body_st, bool few) {
   cudaGraphConditionalHandle cond;
   const bool second = few && h->mg.many_phase();
@@ -582,16 +609,7 @@ static int add_while(psolve_t h, cudaGraph_t graph, double tol, cudaStream_t bod
   if (cudaStreamBeginCaptureToGraph(body_st, body, nullptr, nullptr, 0,
                                     cudaStreamCaptureModeRelaxed) != cudaSuccess)
     return -1;
-  // Several iterations per pass of the WHILE node: a pass costs about 5 us of
-  // its own, an iteration that finds no active plane some 1.3 us a launch, and
-  // half the surplus is spent on average.  Bodies of few launches take 3 (128 x 64
-  // x 128 sphere: 984 us with 1, 948 with 2, 927 with 3, 930 with 4), those
-  // with one level-wide level 2 (FP64 cylinder of 32 x 32: 2524, 2488, 2464, 2458), longer
-  // ones 1 (FP64 sphere of 128 x 64: 7784 with 1, 7789 with 2).  The tail kernel
-  // takes its planes in the iteration that hands them over: 1.
-  const int base = h->mg.base;
-  const int passes = h->mg.tail_planes > 0 ? 1 : (few || base == 0 ? 3 : (base == 1 ? 2 : 1));
-  for (int k = 0; k < passes; ++k) h->mg.loop_body(h->f, h->u, tol, body_st, 1, cond, few);
+  for (int k = 0; k < loop_passes(h, few); ++k) h->mg.loop_body(h->f, h->u, tol, body_st, 1, cond, few);
   cudaGraph_t out;
   return cudaStreamEndCapture(body_st, &out) == cudaSuccess ? 0 : -1;
 }
