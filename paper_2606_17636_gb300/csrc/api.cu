@@ -484,7 +484,8 @@ extern "C" int psolve_get_loops(psolve_t h, psolve_loops* out) {
     for (const auto& leg : *legs) out->few_launches += int(leg.size());
   out->passes = loop_passes(h, false);
   out->few_passes = loop_passes(h, true);
-  out->fused_update = m.base > 0 && m.opt.nu2 > 0 ? 1 : 0;
+  const bool band = m.opt.precision && band_pays(m.lv[0].nr, m.lv[0].nt, m.opt.n_sor, m.max_planes);
+  out->fused_update = m.base > 0 && m.opt.nu2 > 0 && !band ? 1 : 0;
   return PSOLVE_OK;
 }
 

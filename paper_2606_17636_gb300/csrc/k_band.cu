@@ -209,12 +209,12 @@ __global__ void __launch_bounds__(kBandThreads, CPL == 8 ? 2 : 1)
 // march 22 and 143 (the bytes take 15 and 121).  A step is bound by its chain of
 // dependent multiply-adds with 8 to 12 warps an SM.
 constexpr int kAhead = 4;   // row pairs in flight
-template <int NS, bool UPD>
+template <int NS>
 __global__ void __launch_bounds__(kBandThreads, 3)
     k_march(LevelDev L, Batch B, const float2* __restrict__ ein, float2* __restrict__ eout, const float2* __restrict__ f,
-            int tiles, int width, int target, double2* __restrict__ u) {
+            int tiles, int width, int target) {
   constexpr int W = 4 * NS + 2, D = 2 * NS, kPad = 2 * D;
-  constexpr int kRow = UPD ? 8 : 4;    // float4 per lane and row pair: e, f of both rows, and u
+  constexpr int kRow = 4;    // float4 per lane and row pair: e, f of both rows
   // per row aN, aS, T, -D_theta, zero beyond the plane (a zero row stays zero
   // through its relaxation); then every warp's ring
   extern __shared__ float4 rowtab[];
@@ -271,8 +271,7 @@ __global__ void __launch_bounds__(kBandThreads, 3)
       id0[d] = up0[d] = dn0[d] = id1[d] = up1[d] = dn1[d] = 0.f;
     }
     const int x0 = max(r0 - 2 * D, 0), x1 = r1 + 2 * D;   // rows x, x + 1 enter, x - 2 D and the next leave
-    // rows x, x + 1 of e and f (zeros beyond the plane) and the rows of u that
-    // leave with them; every lane reads only its own copies
+    // rows x, x + 1 of e and f (zeros beyond the plane); every lane reads only its own copies
     const float4* ge = reinterpret_cast<const float4*>(ein + base) + size_t(x0) * hr;
     const float4* gf = reinterpret_cast<const float4*>(f + base) + size_t(x0) * hr;
     int fx = x0;
@@ -284,16 +283,6 @@ __global__ void __launch_bounds__(kBandThreads, 3)
       cp_async_v(d + 32, (ok ? ge : reinterpret_cast<const float4*>(ein)) + o, ok);
       cp_async_v(d + 64, ok ? gf : reinterpret_cast<const float4*>(f), ok);
       cp_async_v(d + 96, (ok ? gf : reinterpret_cast<const float4*>(f)) + o, ok);
-      if constexpr (UPD) {
-        const int s0 = fx - 2 * D;
-        if (own && s0 >= r0 && s0 < r1) {
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
-              cp_async_v(d + (4 + 2 * h + c) * 32, reinterpret_cast<const float4*>(u + base + size_t(s0 + h) * nr + c), true);
-        }
-      }
       asm volatile("cp.async.commit_group;\n" ::: "memory");
       ge += 2 * hr;
       gf += 2 * hr;
@@ -359,24 +348,8 @@ __global__ void __launch_bounds__(kBandThreads, 3)
         O[D + s] = fma2(nw[1], fma2(id1[s], r, O[D + s]), O[D + s]);
       }
       if (own && s0 >= r0 && s0 < r1) {
-        if constexpr (UPD) {
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const float2 a = E[W - 1 - h], b = O[W - 1 - h];
-            double2 v = *reinterpret_cast<const double2*>(row + (4 + 2 * h) * 32);
-            double2 w = *reinterpret_cast<const double2*>(row + (5 + 2 * h) * 32);
-            v.x += widen(a.x);
-            v.y += widen(a.y);
-            w.x += widen(b.x);
-            w.y += widen(b.y);
-            double2* o = u + base + size_t(s0 + h) * nr;
-            o[0] = v;
-            o[1] = w;
-          }
-        } else {
-          out[0] = make_float4(E[W - 1].x, E[W - 1].y, O[W - 1].x, O[W - 1].y);
-          out[hr] = make_float4(E[W - 2].x, E[W - 2].y, O[W - 2].x, O[W - 2].y);
-        }
+        out[0] = make_float4(E[W - 1].x, E[W - 1].y, O[W - 1].x, O[W - 1].y);
+        out[hr] = make_float4(E[W - 2].x, E[W - 2].y, O[W - 2].x, O[W - 2].y);
       }
       out += 2 * hr;
     }
@@ -404,20 +377,19 @@ void radial(const LevelDev& L, const Batch& B, const float2* ein, float2* eout, 
       L, B, ein, eout, f, zi ? 1 : 0, n_sor, resident);
 }
 
-template <int NS, bool UPD>
-void march(const LevelDev& L, const Batch& B, const float2* ein, float2* eout, const float2* f, double2* u,
-           cudaStream_t st) {
+template <int NS>
+void march(const LevelDev& L, const Batch& B, const float2* ein, float2* eout, const float2* f, cudaStream_t st) {
   const int pairs = L.nr / 2, tiles = (pairs + 29) / 30, width = (pairs + tiles - 1) / tiles;
   const int resident = sm_count() * 3 * (kBandThreads / 32);
   const long most = long(B.max_planes) * tiles * (L.nt / 8);
   const long warps = most < resident ? most : resident;
-  const size_t sm = (size_t(L.nt) + 8 * NS + (kBandThreads / 32) * kAhead * (UPD ? 8 : 4) * 32) * sizeof(float4);
+  const size_t sm = (size_t(L.nt) + 8 * NS + (kBandThreads / 32) * kAhead * 4 * 32) * sizeof(float4);
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(k_march<NS, UPD>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
+    cudaFuncSetAttribute(k_march<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
     attr = true;
   }
-  k_march<NS, UPD><<<unsigned((warps + kBandThreads / 32 - 1) / (kBandThreads / 32)), kBandThreads, sm, st>>>(L, B, ein, eout, f, tiles, width, resident, u);
+  k_march<NS><<<unsigned((warps + kBandThreads / 32 - 1) / (kBandThreads / 32)), kBandThreads, sm, st>>>(L, B, ein, eout, f, tiles, width, resident);
 }
 
 }  // namespace
@@ -437,18 +409,11 @@ void launch_band_radial(const LevelDev& L, const Batch& B, const float2* ein, fl
   else radial<8>(L, B, ein, eout, f, zero_init, n_sor, st);
 }
 
-void launch_march(const LevelDev& L, const Batch& B, const float2* ein, float2* eout, const float2* f, int n_sor, double2* u,
+void launch_march(const LevelDev& L, const Batch& B, const float2* ein, float2* eout, const float2* f, int n_sor,
                   cudaStream_t st) {
-  if (n_sor == 1) {
-    if (u) march<1, true>(L, B, ein, eout, f, u, st);
-    else march<1, false>(L, B, ein, eout, f, u, st);
-  } else if (n_sor == 2) {
-    if (u) march<2, true>(L, B, ein, eout, f, u, st);
-    else march<2, false>(L, B, ein, eout, f, u, st);
-  } else {
-    if (u) march<3, true>(L, B, ein, eout, f, u, st);
-    else march<3, false>(L, B, ein, eout, f, u, st);
-  }
+  if (n_sor == 1) march<1>(L, B, ein, eout, f, st);
+  else if (n_sor == 2) march<2>(L, B, ein, eout, f, st);
+  else march<3>(L, B, ein, eout, f, st);
 }
 
 }  // namespace ps

@@ -259,7 +259,7 @@ bool band_pays(int nr, int nt, int n_sor, int planes);
 void launch_band_radial(const LevelDev& L, const Batch& B, const float2* ein, float2* eout, const float2* f,
                         bool zero_init, int n_sor, cudaStream_t st);
 void launch_march(const LevelDev& L, const Batch& B, const float2* ein, float2* eout, const float2* f, int n_sor,
-                  double2* u, cudaStream_t st);
+                  cudaStream_t st);
 
 // Several smoothing passes of a level per launch on overlapping windows
 // (k_tile.cu, FP32).
