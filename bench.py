@@ -651,18 +651,17 @@ def launches_per_solve(s, st):
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of full-batch
 # launches on workload 3 (all 129 modes), from the ncu captures of the
 # profiling case (python -m paper_2606_17636_gb300.profile_case
-# --schedule 2,1,2,4,16,2,2 --smooth-first): one k_vsmem launch, one
-# finest-level smoothing cycle (k_rpass2 + k_tpass2) and the first stencil
+# --schedule 2,1,2,4,16,2,2 --smooth-first): one k_vpatch launch, one
+# finest-level smoothing cycle (k_band + k_march) and the first stencil
 # launch of k_residual.  They hold for the kernels as captured; a changed
 # kernel needs a new capture.
-VSMEM_TRAFFIC_BYTES = 13804288 + 1536
-SMOOTH_CYCLE_TRAFFIC_BYTES = 67736064 + 8047872 + 67791616 + 6110720
-RESIDUAL_TRAFFIC_BYTES = 169755136 + 18508544
+VSMEM_TRAFFIC_BYTES = 13771520
+SMOOTH_CYCLE_TRAFFIC_BYTES = 67737344 + 2694656 + 69978624 + 5459712
+RESIDUAL_TRAFFIC_BYTES = 169805568 + 23041280
 # ncu sm__inst_executed_pipe_fp64 (percent of peak, sustained active) of the
-# kernels bound by the FP64 pipe: k_residual and k_fft_fwd from the same
-# capture at 256 x 128 x 256, k_fft_inv and k_boundary at 256 x 128 x 128
-# (the same kernels with 65 mode planes)
-FP64_PIPE_PCT = {"k_residual": 77.5, "k_fft_fwd": 83.8, "k_fft_inv": 82.3, "k_boundary": 87.1}
+# kernels bound by the FP64 pipe: k_residual from the same capture at 256 x
+# 128 x 256, k_boundary at 256 x 128 x 128 (the same kernel, 65 mode planes)
+FP64_PIPE_PCT = {"k_residual": 77.6, "k_boundary": 87.1}
 
 
 def vcycle_flops_per_cell(sched):
@@ -717,10 +716,11 @@ def fp64_peak_tflops(torch):
 
 def fft_roofline(torch, ps, s, fp64_peak, reps=20):
     """The forward azimuthal transform (k_fft_fwd) of the workload, timed
-    alone through psolve_stage_forward with CUDA events.  Work: n_r n_tz / 2
-    complex FFTs of n_phi points (two real rows packed in one), 5 N log2 N
-    flops each, against the measured FP64 GEMM rate: the kernel runs on the
-    FP64 pipe (ncu: FP64_PIPE_PCT)."""
+    alone through psolve_stage_forward with CUDA events.  It works in block
+    fixed point (64-bit integers), off the FP64 pipe, and is bound by integer
+    instructions; reported against HBM (each value read once, each mode written
+    once), with the 5 N log2 N flops of n_r n_tz / 2 packed complex FFTs
+    beside it, whose rate exceeds the FP64 GEMM's."""
     import math
     n_r, n_tz, n_phi = s.grid
     rho = torch.rand((n_r, n_tz, n_phi), dtype=torch.float64, device="cuda")
@@ -735,13 +735,15 @@ def fft_roofline(torch, ps, s, fp64_peak, reps=20):
     torch.cuda.synchronize()
     dt = e0.elapsed_time(e1) / 1e3 / reps
     flops = (n_r * n_tz / 2) * 5 * n_phi * math.log2(n_phi)
-    ach = flops / dt / 1e12
-    return {"kernel": "forward azimuthal transform k_fft_fwd", "bound": "fp64", "achieved": ach,
-            "peak": fp64_peak, "unit": "TFLOP/s", "frac": ach / fp64_peak,
-            "peak_source": "measured: cuBLAS FP64 GEMM 4096^3 on this GPU",
-            "ncu_fp64_pipe_pct": FP64_PIPE_PCT["k_fft_fwd"],
-            "algorithmic_flops_per_launch": flops, "avg_ms": dt * 1e3,
-            "bytes_per_launch": 8.0 * n_r * n_tz * n_phi + 16.0 * n_r * n_tz * (n_phi // 2 + 1)}
+    bytes_ = 8.0 * n_r * n_tz * n_phi + 16.0 * n_r * n_tz * (n_phi // 2 + 1)
+    pk = peaks().get("hbm_gbs")
+    return {"kernel": "forward azimuthal transform k_fft_fwd (block fixed point)", "bound": "hbm",
+            "achieved": bytes_ / dt / 1e9, "peak": pk, "unit": "GB/s",
+            "frac": (bytes_ / dt / 1e9 / pk) if pk else None,
+            "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)",
+            "tflops": flops / dt / 1e12, "fp64_gemm_tflops": fp64_peak,
+            "algorithmic_flops_per_launch": flops, "avg_ms": dt * 1e3, "bytes_per_launch": bytes_,
+            "note": "integer-instruction bound; each timed call also allocates its result and synchronises"}
 
 
 def residual_roofline(torch, ps, s, stream, fp64_peak, reps=20):
@@ -789,8 +791,9 @@ def residual_roofline(torch, ps, s, stream, fp64_peak, reps=20):
 
 
 def vcycle_roofline(torch, ps, s, stream):
-    """The dominant kernel: the fused coarse V-cycle (k_vsmem, one block per
-    mode plane, levels held in shared memory), all modes, timed alone
+    """The dominant kernel: the fused coarse V-cycle (k_vpatch, one block per
+    mode plane, its first level in registers and the rest in shared memory;
+    k_vsmem where that level has another size), all modes, timed alone
     through psolve_stage_vcycle with CUDA events on the library's stream.
     Algorithmic work per launch: M x sum over the fused smoothed levels of
     cells x vcycle_flops_per_cell(schedule) FP32 flops, plus the separable solve
@@ -824,7 +827,7 @@ def vcycle_roofline(torch, ps, s, stream):
     # Thomas solves along r (FP64)
     flops = M * (cells * vcycle_flops_per_cell(s.schedule()) + 8 * cr * ct * ct + 10 * cr * ct)
     ach = flops / dt / 1e12
-    return {"kernel": "fused coarse V-cycle k_vsmem (levels %d..%d in shared memory, all %d modes)"
+    return {"kernel": "fused coarse V-cycle k_vpatch (levels %d..%d on chip, all %d modes)"
                       % (lev, s.n_levels - 1, M),
             "bound": "alu", "achieved": ach, "peak": peak32, "unit": "TFLOP/s",
             "frac": ach / peak32,
@@ -859,7 +862,7 @@ def smoother_roofline(torch, ps, s, stream):
     bytes_ = 48.0 * M * n_tz * n_r
     pk = peaks().get("hbm_gbs")
     ach = bytes_ / dt / 1e9
-    return {"kernel": "finest-level smoothing cycle (k_rpass2 + k_tpass2, FP32, all modes)",
+    return {"kernel": "finest-level smoothing cycle (FP32, both directions, all modes)",
             "bound": "hbm", "achieved": ach, "peak": pk, "unit": "GB/s",
             "frac": (ach / pk) if pk else None, "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)",
             "traffic": SMOOTH_CYCLE_TRAFFIC_BYTES if M == 129 and (n_r, n_tz) == (256, 128) else None,

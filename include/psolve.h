@@ -293,7 +293,8 @@ int psolve_get_loops(psolve_t h, psolve_loops* out);
  * or three, and a few SOR sweeps per line); it changes the convergence rate,
  * not the converged answer.  The tile shapes of the level-wide smoothing
  * passes change only how lines are grouped into thread blocks: every tile
- * shape gives bitwise the same result. */
+ * shape gives bitwise the same result.  FP32 levels of 1.5 M cells and more over
+ * all planes are relaxed in registers and ignore them. */
 typedef struct {
   int nu_pre, nu_post; /* smoothing cycles before / after coarse correction, 1..8 */
   int n_sor;           /* SOR sweeps per line relaxation, 1..8                    */
