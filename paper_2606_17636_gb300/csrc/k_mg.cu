@@ -9,6 +9,7 @@
 #include <type_traits>
 
 #include "lines.cuh"
+#include "residual_split.h"
 
 namespace ps {
 
@@ -346,9 +347,6 @@ __device__ __forceinline__ Sum4 sum_of(const SqPart& q) {
 }
 
 constexpr int kFlatItems = 256;
-// Blocks that 1024-cell items must give (two an SM); with fewer, 256-cell items
-// use more SMs (17 planes of 32 x 32 cells, FP64: 8.2 us, 14.2 with 17 blocks).
-constexpr int kWideBlocks = 304;
 
 // The residual work items of one launch.  ZERO: u = 0 on the first
 // iteration, so r = f and |r|^2 = |f|^2 (no stencil); CPT: cells per thread
@@ -362,11 +360,12 @@ __device__ __forceinline__ void residual_items(const LevelDev& L, const Batch& B
                                                int* cnt, int bpp, const RetireArgs& ra,
                                                const double* __restrict__ ctab,
                                                const double* __restrict__ dtab, int nact,
-                                               bool want_f, SqPart* sh, int* flag, int* scan) {
+                                               const ResidualSplit& split, bool want_f, SqPart* sh,
+                                               int* flag, int* scan) {
   const int nr = L.nr, nt = L.nt, n = nr * nt;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = int(blockDim.x >> 5);
-  const int ipp = (bpp + CPT - 1) / CPT;   // items per plane
-  for (int w = blockIdx.x; w < nact * ipp; w += gridDim.x) {
+  const int ipp = split.items_per_plane;
+  for (int w = blockIdx.x; w < split.items; w += gridDim.x) {
     const int k = w / ipp, bx = w - k * ipp;
     const int p = B.act[k];
     const int slot = B.slot ? B.slot[p] : p;
@@ -446,7 +445,7 @@ __device__ __forceinline__ void residual_items(const LevelDev& L, const Batch& B
           psum[p] = sum_of(q);
           cnt[p] = 0;
           __threadfence();
-          flag[1] = (atomicAdd(ra.gcnt, 1) == nact - 1);
+          flag[1] = (atomicAdd(ra.gcnt, 1) == nact + split.waiting - 1);
         }
       }
       __syncthreads();
@@ -465,43 +464,51 @@ template <typename T>
 __global__ void __launch_bounds__(256, 5) k_residual(LevelDev L, Batch B, const double2* __restrict__ f,
                                                   const double2* __restrict__ u,
                                                   vec2_t<T>* __restrict__ r, SqPart* part,
-                                                  Sum4* psum, int* cnt, int bpp, RetireArgs ra,
+                                                  Sum4* psum, int* cnt, int bpp, int sms, RetireArgs ra,
                                                   const double* __restrict__ ctab,
                                                   const double* __restrict__ dtab) {
   __shared__ SqPart sh[8];
   __shared__ int flag[2];
   __shared__ int scan[256];
   // nact is read once: the retiring block rewrites it only after every work
-  // item of this launch has been summed
+  // item of this launch has been summed.  A block that starts after that finds no
+  // item with the smaller count either (residual_split).
   const int nact = *B.nact;
+  const ResidualSplit split = residual_split(nact, bpp, int(gridDim.x), sms);
   const bool want_f = *ra.S.iter == 0;     // |f| is needed on the first iteration only
   // from a zero initial guess the first defect is f itself (no stencil)
   const bool r_is_f = want_f && ra.zero_guess;
-  // Work items of CPT x 256 cells: with many cells active the per-item
-  // reduction, fence and arrival count are paid once per 1024 cells; with few
-  // cells every item is 256 cells, spreading a plane's FP64 work over more
-  // SMs.  bpp (the caller's) is the item count for CPT = 1.  Up to kFlatItems
+  // bpp (the caller's) counts 256-cell items.  Up to kFlatItems
   // such items one arrival counter serves all planes and the last block sums every
   // plane's items (a warp per plane) and retires: a round of fence, atomic and
   // reload less (one plane of 128 x 64 cells: 7.9 us, 9.8 before; with up to
   // 4096 items 10 planes of 256 x 128 took 24.5 us, 20.3 with a counter per
   // plane: arrivals at one address queue).  48 registers (5 blocks an SM): with
   // 56 the full batch of 256 x 128 took 111 us, 104 so.
-  const bool flat = nact * bpp <= kFlatItems && nact <= int(blockDim.x);
+  const bool flat = !split.wide && split.items <= kFlatItems && nact <= int(blockDim.x);
   auto items = [&](auto zero, auto cpt, auto fl) {
     residual_items<T, decltype(zero)::value, decltype(cpt)::value, decltype(fl)::value>(
-        L, B, f, u, r, part, psum, cnt, bpp, ra, ctab, dtab, nact, want_f, sh, flag, scan);
+        L, B, f, u, r, part, psum, cnt, bpp, ra, ctab, dtab, nact, split, want_f, sh, flag, scan);
   };
   using one = std::integral_constant<int, 1>;
   using four = std::integral_constant<int, 4>;
-  const bool wide = nact >= 16 && nact * bpp >= 4 * kWideBlocks;
   if (r_is_f) {
-    if (wide) items(std::true_type{}, four{}, std::false_type{});
+    if (split.wide) items(std::true_type{}, four{}, std::false_type{});
     else items(std::true_type{}, one{}, std::false_type{});
   } else {
-    if (wide) items(std::false_type{}, four{}, std::false_type{});
+    if (split.wide) items(std::false_type{}, four{}, std::false_type{});
     else if (flat) items(std::false_type{}, one{}, std::true_type{});
     else items(std::false_type{}, one{}, std::false_type{});
+  }
+  if (split.wide && int(blockIdx.x) >= split.items) {   // no item: the arrival alone, after the count was read
+    if (threadIdx.x == 0) flag[1] = (atomicAdd(ra.gcnt, 1) == nact + split.waiting - 1);
+    __syncthreads();
+    if (flag[1]) {
+      __threadfence();
+      retire_block(const_cast<int*>(B.act), const_cast<int*>(B.nact), psum, ra.S, ra.tol, ra.max_cycles, ra.stagnation,
+                   ra.use_cond, ra.handle, scan, ra.tail_planes, ra.host, RetireHint{});
+      if (threadIdx.x == 0) *ra.gcnt = 0;
+    }
   }
 }
 
@@ -510,8 +517,8 @@ void launch_residual(const LevelDev& L, const Batch& B, const double2* f, const 
                      vec2_t<T>* r, SqPart* part, Sum4* psum, int* cnt, const RetireArgs& ra,
                      cudaStream_t st, const double* ctab, const double* dtab) {
   const int bpp = residual_blocks(L.nr, L.nt);
-  k_residual<T><<<work_grid(long(bpp) * B.max_planes), 256, 0, st>>>(L, B, f, u, r, part, psum,
-                                                                       cnt, bpp, ra, ctab, dtab);
+  k_residual<T><<<work_grid(long(bpp) * B.max_planes), 256, 0, st>>>(
+      L, B, f, u, r, part, psum, cnt, bpp, sm_count(), ra, ctab, dtab);
 }
 
 // ---------------------------------------------------------------------------
