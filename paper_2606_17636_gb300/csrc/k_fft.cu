@@ -10,9 +10,10 @@
 // for 256 x 128 rows of 256 values (152 us of pipe time at best for
 // 5 N log2 N operations), where the bytes take 20 us.  In fixed point an
 // addition is two integer instructions and a twiddle product twelve 32-bit
-// multiplies; the same transforms take 70 and 79 us (ncu), bound by the issue
-// of 44 and 55 million warp instructions (integer ALU pipe 52-59 % busy, 16
-// warps an SM at 128 registers).
+// multiplies; the same transforms take 59 and 78 us, bound by the issue of warp
+// instructions (16 warps an SM at 128 registers).  Zero times a twiddle is zero, so
+// that modes which cancel exactly, those of rows constant or periodic along phi,
+// come out as zeros and retire at their first residual.
 //
 // Scaling: a row's values are aligned to its largest exponent (a power of two
 // each, so scaling a row scales its spectrum exactly).  Every partial sum of a
@@ -51,30 +52,32 @@ struct Z {
 __device__ __forceinline__ Z operator+(Z a, Z b) { return Z{a.x + b.x, a.y + b.y}; }
 __device__ __forceinline__ Z operator-(Z a, Z b) { return Z{a.x - b.x, a.y - b.y}; }
 
-// Constants w = (h 2^31 + l) 2^-61, |w| <= 1.
-constexpr int kR_h = 759250124, kR_l = 2134625425;   // sqrt(1/2)
-constexpr int kC_h = 992008094, kC_l = 848119337;    // cos(pi / 8)
-constexpr int kS_h = 410903206, kS_l = 1465168233;   // sin(pi / 8)
+// Constants w = (h 2^32 + l) 2^-62, |w| <= 1, -2^31 <= l < 2^31.
+constexpr int kR_h = 759250125, kR_l = -25716447;   // sqrt(1/2)
+constexpr int kC_h = 992008094, kC_l = 1696238673;   // cos(pi / 8)
+constexpr int kS_h = 410903207, kS_l = -1364630830;   // sin(pi / 8)
 
-// x = h 2^31 + l with 0 <= l < 2^31.
-__device__ __forceinline__ int hi31(i64 x) { return int(x >> 31); }
-__device__ __forceinline__ int lo31(i64 x) { return int(x & 0x7fffffff); }
+// x = h 2^32 + l with the same range of l: one instruction, l being the low word as
+// it stands (with l unsigned, the product left out below had a mean to add: nonzero
+// for x = 0, and 66 and 84 us for the transforms above).
+__device__ __forceinline__ int hi32(i64 x) { return int(x >> 32) + int(unsigned(x) >> 31); }
+__device__ __forceinline__ int lo32(i64 x) { return int(unsigned(x)); }
 __device__ __forceinline__ i64 mulw(int a, int b) { return i64(a) * i64(b); }
 
-// x w for |x| < 2^62: the product of the low halves (below two units) is
-// replaced by its mean over x's, l / 2 of the middle products' unit.
+// x w for |x| < 2^62, rounded but for the product of the low halves, which is
+// left out: at most one unit, of either sign alike, and zero where x has no low
+// half, so that zero times w is zero.
 __device__ __forceinline__ i64 mulq(i64 x, int h, int l) {
-  const int xh = hi31(x), xl = lo31(x);
-  return (mulw(xh, h) << 1) + ((mulw(xh, l) + mulw(xl, h) + ((1 << 29) + (l >> 1))) >> 30);
+  const int xh = hi32(x), xl = lo32(x);
+  return (mulw(xh, h) << 2) + ((mulw(xh, l) + mulw(xl, h) + (1 << 29)) >> 30);
 }
 // z (wr + i wi) for |z.x|, |z.y| < 2^61 (the halves' sums stay below 2^63).
 __device__ __forceinline__ Z mulz(Z z, int rh, int rl, int ih, int il) {
-  const int xh = hi31(z.x), xl = lo31(z.x), yh = hi31(z.y), yl = lo31(z.y);
+  const int xh = hi32(z.x), xl = lo32(z.x), yh = hi32(z.y), yl = lo32(z.y);
   const i64 a = mulw(xh, rh) - mulw(yh, ih), b = mulw(xh, ih) + mulw(yh, rh);
   const i64 c = mulw(xh, rl) + mulw(xl, rh) - mulw(yh, il) - mulw(yl, ih);
   const i64 d = mulw(xh, il) + mulw(xl, ih) + mulw(yh, rl) + mulw(yl, rh);
-  const int u = rl >> 1, v = il >> 1;
-  return Z{(a << 1) + ((c + ((1 << 29) + u - v)) >> 30), (b << 1) + ((d + i64(1 << 29) + i64(u) + i64(v)) >> 30)};
+  return Z{(a << 2) + ((c + (1 << 29)) >> 30), (b << 2) + ((d + (1 << 29)) >> 30)};
 }
 
 // SIGN < 0: e^{-2 pi i}, SIGN > 0: e^{+2 pi i}.
@@ -527,7 +530,7 @@ void inverse(const double2* fh, double* phi, int nr, int nt, const FftTables& ta
 }  // namespace
 
 // Twiddles of both transforms of length N as (h, l) pairs of cos and sin in
-// units of 2^-61; the forward's first pass carries the scale's mantissa.
+// units of 2^-62; the forward's first pass carries the scale's mantissa.
 // Lengths of one pass have no twiddles: the output takes the scale.  A scale
 // that is not finite gives NaN.
 std::vector<int4> fft_tables(int N, double scale, FftTables* t, size_t* inv_at) {
@@ -539,12 +542,11 @@ std::vector<int4> fft_tables(int N, double scale, FftTables* t, size_t* inv_at) 
   t->post = scale;
   if (!fold) ms = 1.0;
   std::vector<int4> out;
-  const long double pi = 3.14159265358979323846264338327950288L, unit = 2305843009213693952.0L;   // 2^61
+  const long double pi = 3.14159265358979323846264338327950288L, unit = 4611686018427387904.0L;   // 2^62
   auto part = [&](long double x, int& h, int& l) {
     const i64 q = i64(std::floor(x * unit + 0.5L));
-    const i64 hi = (q - (q & 0x7fffffffll)) / 2147483648ll;   // floor
-    h = int(hi);
-    l = int(q & 0x7fffffffll);
+    l = int(static_cast<unsigned>(q));   // the low half with its sign
+    h = int((q - l) / 4294967296ll);
   };
   for (int dir = 0; dir < 2; ++dir) {
     if (dir == 1) *inv_at = out.size();

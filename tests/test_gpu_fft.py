@@ -131,3 +131,41 @@ def test_ragged_slabs_equal_the_whole_grid(ps, n, rows):
     gp = s.stage_inverse_rows(f[:, :, :rows].contiguous())
     assert torch.equal(gp[:even], g[:even]) and torch.allclose(gp, g[:rows], rtol=0, atol=1e-12)
     s.close()
+
+
+@pytest.mark.parametrize("n", LENGTHS)
+def test_exact_zeros_of_periodic_rows(ps, n):
+    """Differences of equal values are zero and stay zero through the twiddles:
+    rows constant along phi have no modes above m = 0, rows of period n / p only
+    every p-th one; the inverse of such spectra has rows of that period."""
+    rng = np.random.default_rng(n)
+    s = _solver(ps, n)
+    for p in (2, 4, n):
+        if p > n // 2 and p != n:
+            continue
+        x = np.tile(rng.standard_normal((32, 16, n // p)) + 3.0, p)
+        f = s.stage_forward(torch.from_numpy(x).cuda())
+        others = torch.arange(n // 2 + 1, device="cuda") % p != 0
+        assert torch.count_nonzero(f[others]) == 0
+        ref = np.fft.rfft(x, axis=2).transpose(2, 1, 0) * (4 * np.pi / n)
+        assert np.abs(f.cpu().numpy() - ref).max() <= 1e-14 * np.abs(ref).max()
+        g = s.stage_inverse(f)
+        assert torch.equal(g, g[:, :, : n // p].repeat(1, 1, p))
+    s.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("graph", [False, True])
+def test_modes_of_an_axisymmetric_density_retire_at_once(ps, precision, graph):
+    """A density without phi dependence: every m > 0 is an exact zero and takes no
+    cycle in either solve, and the potential does not depend on phi."""
+    sp = workloads.spec(workloads.SPHERICAL, 64, 32, 32, workloads.LOG, 0.1, 10.0)
+    s = ps.Solver.from_spec(sp, precision=precision, use_graph=graph)
+    rho = torch.rand((64, 32, 1), dtype=torch.float64, device="cuda").expand(64, 32, 32).contiguous()
+    phi, rc = s.solve(rho, tol=1e-9)
+    assert rc == ps.OK
+    st = s.stats()
+    assert st["cycles_psi"][0] > 0 and st["cycles_phi"][0] > 0
+    assert not any(st["cycles_psi"][1:]) and not any(st["cycles_phi"][1:])
+    assert torch.equal(phi, phi[:, :, :1].expand_as(phi))
+    s.close()
