@@ -10,7 +10,7 @@
 // for 256 x 128 rows of 256 values (152 us of pipe time at best for
 // 5 N log2 N operations), where the bytes take 20 us.  In fixed point an
 // addition is two integer instructions and a twiddle product twelve 32-bit
-// multiplies; the same transforms take 59 and 78 us, bound by the issue of warp
+// multiplies; the same transforms take 61 and 79 us, bound by the issue of warp
 // instructions (16 warps an SM at 128 registers).  Zero times a twiddle is zero, so
 // that modes which cancel exactly, those of rows constant or periodic along phi,
 // come out as zeros and retire at their first residual.
@@ -18,15 +18,17 @@
 // Scaling: a row's values are aligned to its largest exponent (a power of two
 // each, so scaling a row scales its spectrum exactly).  Every partial sum of a
 // transform is bounded by the sum of the magnitudes that enter it, so a row is
-// scaled to bring that sum (formed in FP32, rounded up) just below 2^60: no
-// step can overflow, a row with one dominant value keeps all its 53 bits with
-// room below, and a flat row of N values keeps 60 - log2 N.  Above 256 values
-// the first pass is scaled by the smaller bound radix x maximum and the
-// twiddle products shift the rest out.  What error remains is the rounding of
-// the values, the twiddle products and the final one to FP64; relative to a
-// row's 2-norm it is below that of the FP64 transform (both against extended
-// precision; 256 values, white noise: 1.0e-16 and 3.3e-16).  A row pair with an
-// infinity or NaN gives NaN, as FP64 arithmetic does.
+// scaled to bring that sum (formed in FP32, rounded up) just below 2^61: no
+// step can overflow, and a row with one dominant value keeps all its 53 bits with
+// room below.  A flat row of N values would keep 61 - log2 N; from 128 values on
+// the first pass is scaled by the smaller bound radix x maximum instead and the
+// twiddle products shift the rest out, so that flat rows keep all 53 too.  What
+// error remains is that of the twiddle products and the final rounding to FP64.
+// Relative to a row's 2-norm, against extended precision, here and in FP64 radix 2
+// (rms over 400 rows of 256 values, in 1e-17): white noise 5.3 and 34, a bump 5.3
+// and 33, 1 + 1 % noise 4.5 and 14, 1 + 0.01 cos 1.6 and 2.8, constant rows 5.0
+// and 4.9 (the final rounding alone); the inverse 4.1 to 5.5 and 4.1 to 48.
+// A row pair with an infinity or NaN gives NaN, as FP64 arithmetic does.
 //
 // Work split: N / 16 threads per row pair, 16 values in a thread's registers;
 // passes of radix 16, 8 or 4 with one exchange through shared memory between
@@ -59,19 +61,20 @@ constexpr int kS_h = 410903207, kS_l = -1364630830;   // sin(pi / 8)
 
 // x = h 2^32 + l with the same range of l: one instruction, l being the low word as
 // it stands (with l unsigned, the product left out below had a mean to add: nonzero
-// for x = 0, and 66 and 84 us for the transforms above).
+// for x = 0, and 66 and 84 us against 59 and 78 for the transforms above).
 __device__ __forceinline__ int hi32(i64 x) { return int(x >> 32) + int(unsigned(x) >> 31); }
 __device__ __forceinline__ int lo32(i64 x) { return int(unsigned(x)); }
 __device__ __forceinline__ i64 mulw(int a, int b) { return i64(a) * i64(b); }
 
-// x w for |x| < 2^62, rounded but for the product of the low halves, which is
+// x w for |x| < 2^62.5, rounded but for the product of the low halves, which is
 // left out: at most one unit, of either sign alike, and zero where x has no low
 // half, so that zero times w is zero.
 __device__ __forceinline__ i64 mulq(i64 x, int h, int l) {
   const int xh = hi32(x), xl = lo32(x);
   return (mulw(xh, h) << 2) + ((mulw(xh, l) + mulw(xl, h) + (1 << 29)) >> 30);
 }
-// z (wr + i wi) for |z.x|, |z.y| < 2^61 (the halves' sums stay below 2^63).
+// z (wr + i wi) for |z| <= 2^62 and |w| <= 1: the sums of the mixed products stay
+// below 2^62 + 2^61.5 (high half of z times low half of w, and the other way round).
 __device__ __forceinline__ Z mulz(Z z, int rh, int rl, int ih, int il) {
   const int xh = hi32(z.x), xl = lo32(z.x), yh = hi32(z.y), yl = lo32(z.y);
   const i64 a = mulw(xh, rh) - mulw(yh, ih), b = mulw(xh, ih) + mulw(yh, rh);
@@ -207,7 +210,8 @@ __device__ __forceinline__ void passes(Z (&v)[values(N)], longlong2* S, const in
 #pragma unroll
   for (int b = 0; b < NB; ++b) butterfly<R, SIGN>(v + b * R);
   if constexpr (!last) {
-    const int first = min(D, ilog(radix(N, 1)));
+    // two passes: all of D here; three: what the second pass does not need
+    const int first = radix(N, 2) == 1 ? D : min(D, ilog(radix(N, 1)));
     const int s = P == 0 ? first : D - first;
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
@@ -216,7 +220,7 @@ __device__ __forceinline__ void passes(Z (&v)[values(N)], longlong2* S, const in
       for (int r = 0; r < R; ++r) {
         const int4 w = __ldg(tw + table_at(N, P) + r * L + g % L);
         Z z = mulz(v[b * R + r], w.x, w.y, w.z, w.w);
-        if constexpr (N > 256) z = Z{shr_round(z.x, s), shr_round(z.y, s)};
+        if constexpr (N >= 128) z = Z{shr_round(z.x, s), shr_round(z.y, s)};
         v[b * R + r] = z;
       }
     }
@@ -249,7 +253,7 @@ __device__ __forceinline__ i64 to_fixed(u64 b, int em, int sh) {
   const u64 m = r > 61 ? 0ull : (((significand(b) << 8) >> r) + 1ull) >> 1;
   return i64(b) < 0 ? -i64(m) : i64(m);
 }
-// v 2^e with |v| <= 2^62, rounded to nearest even: in integer
+// v 2^e with |v| < 2^63, rounded to nearest even: in integer
 // arithmetic where the value has more than 32 bits and e (safe: |e| < 900)
 // keeps the result normal, else through the FP64 pipe.
 __device__ __forceinline__ bool safe_exponent(int e) { return e > -900 && e < 900; }
@@ -297,8 +301,9 @@ __device__ __forceinline__ float row_sum(float x, int* red) {
 
 // Left shift of a row's values from units of 2^(em - 1075), given the sum of
 // their magnitudes in units of 2^(em - 1023), and the bits by which the whole
-// sum then exceeds 2^60 (lengths above 256: the first pass only meets radix
-// values below 4 2^(em - 1023); else 0).
+// sum then exceeds 2^61 (from 128 values on: the first pass only meets radix
+// values below 2^(em - 1022) of each row, in the inverse transform with a factor
+// sqrt(2) for their two parts, 2^61.5 in all; else 0).
 struct RowScale {
   int sh, drop;
 };
@@ -307,12 +312,12 @@ __device__ __forceinline__ RowScale row_scale(float sum) {
   // at most 1e-4 too small, whatever rounding down the magnitudes met
   const int top = int(__float_as_uint(fmaxf(sum, 1.f) * 1.0001f) >> 23) - 127;   // sum < 2^(top + 1)
   RowScale s;
-  s.sh = 7 - top;
+  s.sh = min(8 - top, 7);
   s.drop = 0;
-  if constexpr (N > 256) {
-    constexpr int cap = ilog(radix(N, 0)) + 1;   // radix values of two components each
+  if constexpr (N >= 128) {
+    constexpr int cap = ilog(radix(N, 0)) + 1;
     if (top > cap) {
-      s.sh = 7 - cap;
+      s.sh = 8 - cap;
       s.drop = top - cap;
     }
   }
@@ -320,8 +325,7 @@ __device__ __forceinline__ RowScale row_scale(float sum) {
 }
 
 // Marks in place of a row's exponent: a pair with an infinity or NaN, and a row
-// of zeros (whose transform is exactly zero; the rounding of a transform of
-// zeros is not).
+// of zeros (whose transform is exactly zero beside another row's rounding errors).
 constexpr int kBadRow = INT_MAX, kZeroRow = INT_MIN;
 __device__ __forceinline__ double from_row(i64 v, int e) {
   if (e == kBadRow) return __longlong_as_double(0x7ff8000000000000ll);

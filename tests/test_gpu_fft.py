@@ -169,3 +169,52 @@ def test_modes_of_an_axisymmetric_density_retire_at_once(ps, precision, graph):
     assert not any(st["cycles_psi"][1:]) and not any(st["cycles_phi"][1:])
     assert torch.equal(phi, phi[:, :, :1].expand_as(phi))
     s.close()
+
+
+def _rms(got, ref):
+    return float(np.sqrt(((np.abs(got - ref) ** 2).sum(1) / (np.abs(ref) ** 2).sum(1)).mean()))
+
+
+def _rounded(ref):
+    out = np.empty_like(ref)
+    if np.iscomplexobj(ref):
+        out.real, out.imag = ref.real.astype(np.float64), ref.imag.astype(np.float64)
+    else:
+        out[...] = ref.astype(np.float64)
+    return out
+
+
+@pytest.mark.parametrize("n", [64, 128, 256, 512, 1024])
+@pytest.mark.parametrize("kind", ["cosine", "constant", "noise", "spike"])
+def test_flat_rows_and_spectra_keep_53_bits(ps, n, kind):
+    """Rows nearly constant along phi (forward) and spectra of equal magnitudes
+    (inverse, a spike): the rounding of the exact result to FP64, and per output
+    two units of 2^-60 of the row's sum of magnitudes.  That sum is the norm of a
+    flat row's spectrum, and up to sqrt(2) times that of a spike, so relative to
+    the norm two units of sqrt(n) 2^-60, times sqrt(2) for the spike."""
+    rng = np.random.default_rng(n)
+    s = _solver(ps, n)
+    ph = (np.arange(n) + 0.5) * 2 * np.pi / n
+    shape = (32, 16, 1)
+    rows = rng.choice(32 * 16, 64, replace=False)
+    units = 2 * np.sqrt(n) * 2.0 ** -60
+    if kind == "spike":
+        k = np.exp(-2j * np.pi * np.arange(n // 2 + 1) * rng.integers(0, n, shape) / n) * rng.uniform(1, 2, shape)
+        g = s.stage_inverse(torch.from_numpy(np.ascontiguousarray(k.transpose(2, 1, 0))).cuda()).cpu().numpy()
+        h = k.reshape(-1, n // 2 + 1)[rows].astype(np.clongdouble)
+        h[:, 0], h[:, -1] = h[:, 0].real, h[:, -1].real
+        full = np.concatenate([h, np.conj(h[:, 1:-1][:, ::-1])], axis=1)
+        ref = _dft(full.real, n, 1)[0] - _dft(full.imag, n, 1)[1]
+        got = g.reshape(-1, n)[rows]
+        units *= np.sqrt(2.0)
+    else:
+        c = rng.uniform(1, 2, shape)
+        x = {"cosine": 1.0 + 0.01 * np.cos(ph * rng.integers(1, 4, shape) + rng.uniform(0, 6, shape)),
+             "constant": c * np.ones(n), "noise": c * (1.0 + 0.01 * rng.standard_normal((32, 16, n)))}[kind]
+        f = s.stage_forward(torch.from_numpy(x).cuda()).cpu().numpy().transpose(2, 1, 0)
+        co, si = _dft(x.reshape(-1, n)[rows].astype(np.longdouble), n, -1)
+        ref = (co + 1j * si)[:, : n // 2 + 1] * np.longdouble(4 * np.pi * 1.0 / n)
+        got = f.reshape(-1, n // 2 + 1)[rows]
+    bound = np.hypot(_rms(_rounded(ref), ref), units)
+    assert _rms(got, ref) <= bound, (_rms(got, ref), bound)
+    s.close()
