@@ -282,7 +282,7 @@ static int create_impl(psolve_t* out, const psolve_desc* din, int nd) {
     s->iter = static_cast<int*>(h->A.get(sizeof(int)));
   }
   h->d_worst = static_cast<int*>(h->A.get(sizeof(int)));
-  if (!h->u || !h->f || !d_tw || !h->gt || !h->theta || !h->d_worst || !h->sf.iter) {
+  if (h->A.failed) {
     h->A.release_all();
     return fail(PSOLVE_ERR_NOMEM, "out of device memory");
   }

@@ -41,7 +41,7 @@ static bool green(Arena& A, int geometry, int N, int M, double G, int deriv,
   g.geometry = geometry; g.N = N; g.M = M; g.deriv = deriv; g.G = G;
   g.npairs = long(xt.size());
   g.xt = up(A, xt); g.yt = up(A, yt); g.xs = up(A, xs); g.ys = up(A, ys);
-  if (!g.xt || !g.yt || !g.xs || !g.ys) return false;
+  if (A.failed) return false;   // these, or what the caller passes in
   g.cosk = cosk; g.out = out; g.mstride = mstride; g.pstride = pstride;
   g.scale = scale; g.scale_mod = scale_mod;
   launch_green(g, st);
@@ -142,7 +142,7 @@ static bool build_extended(const PlaneGeo& g, const Law& rlaw, const Law& tlaw,
   if (!mg.init(A, ext, true, modes, slot, int(chunk), o, err)) return false;
   double2* u = static_cast<double2*>(A.get(sizeof(double2) * cells * chunk));
   double2* f = static_cast<double2*>(A.get(sizeof(double2) * cells * chunk));
-  if (!u || !f) { err = "out of device memory (DGF planes)"; return false; }
+  if (A.failed) { err = "out of device memory (DGF planes)"; return false; }
   for (long p0 = 0; p0 < total; p0 += chunk) {
     const int np = int(std::min<long>(chunk, total - p0));
     for (int p = 0; p < np; ++p) slot[p] = int((p0 + p) / ea.npairs);
@@ -308,7 +308,7 @@ static bool build_aux(const PlaneGeo& g, const Law& rlaw, const Law& tlaw,
   a.tcell_i = up(A, ti); a.tcell_j = up(A, tj);
   a.gt = gt;
   a.fail = static_cast<int*>(A.get(sizeof(int)));
-  if (!a.fail || !a.win || !a.tlist) { err = "out of device memory (DGF windows)"; return false; }
+  if (A.failed) { err = "out of device memory (DGF windows)"; return false; }
   cudaMemsetAsync(a.fail, 0, sizeof(int), st);
   launch_aux_cg(a, M * nb, max_cells, st);
   int fails = 0;

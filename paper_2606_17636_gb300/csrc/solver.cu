@@ -27,6 +27,8 @@ void* Arena::get(size_t n) {
   if (p) {
     blocks.push_back(p);
     bytes += n;
+  } else {
+    failed = true;
   }
   return p;
 }
@@ -334,6 +336,7 @@ bool MGSolver::init(Arena& A, const PlaneGeo& fine, bool neumann, const std::vec
     base = nl - 1;
     if (!build_vsmem(A, base, int(modes.size()), vsb, err)) return false;
   }
+  if (A.failed) { err = "out of device memory"; return false; }
   if (!opt.precision) {
     // FP64 smoothing: inverse diagonals per mode and cell of the levels on the
     // line passes, where they take at most an eighth of the free memory (the
@@ -345,7 +348,10 @@ bool MGSolver::init(Arena& A, const PlaneGeo& fine, bool neumann, const std::vec
         const size_t bytes = sizeof(double) * modes.size() * size_t(lv[l].nr) * lv[l].nt;
         double* a = static_cast<double*>(A.get(bytes));
         double* b = static_cast<double*>(A.get(bytes));
-        if (!a || !b) break;
+        if (!a || !b) {   // the passes do without
+          A.failed = false;
+          break;
+        }
         launch_inverse_diagonal(lv[l], d_s2, int(modes.size()), a, b, 0);
         lv[l].idr = a;
         lv[l].idt = b;
@@ -361,7 +367,10 @@ bool MGSolver::init(Arena& A, const PlaneGeo& fine, bool neumann, const std::vec
       e2[l] = A.get(size_t(mp) * lv[l].nr * lv[l].nt * vb);
       if (!e2[l]) tmp2 = nullptr;
     }
-    if (!tmp2) cudaGetLastError();
+    if (!tmp2) {
+      A.failed = false;
+      cudaGetLastError();
+    }
     plan_tiles();
   }
   const int nblk = residual_blocks(lv[0].nr, lv[0].nt);
@@ -378,7 +387,7 @@ bool MGSolver::init(Arena& A, const PlaneGeo& fine, bool neumann, const std::vec
   d_cont = static_cast<int*>(A.get(sizeof(int)));
   d_fmax2 = static_cast<double*>(A.get(sizeof(double)));
   d_gcnt = static_cast<int*>(A.get(sizeof(int)));
-  if (!d_fmax2 || !d_cnt || !d_gcnt) { err = "out of device memory"; return false; }
+  if (A.failed) { err = "out of device memory"; return false; }
   cudaMemset(d_cnt, 0, sizeof(int) * mp);
   cudaMemset(d_gcnt, 0, sizeof(int));
   if (cudaMallocHost(&h_cont, kFlags * sizeof(int)) != cudaSuccess) { err = "pinned allocation failed"; return false; }
@@ -455,7 +464,7 @@ bool MGSolver::init(Arena& A, const PlaneGeo& fine, bool neumann, const std::vec
     }
     tl.titer = static_cast<int*>(A.get(2 * sizeof(int)));
     tl.tdone = tl.titer ? tl.titer + 1 : nullptr;
-    if (!d_tail_tabs || !tl.titer) { err = "out of device memory"; return false; }
+    if (A.failed) { err = "out of device memory"; return false; }
     cudaMemset(tl.titer, 0, 2 * sizeof(int));
     prepare_tail();
   }

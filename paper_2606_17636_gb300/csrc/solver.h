@@ -14,6 +14,7 @@ struct Arena {
   void* user = nullptr;
   std::vector<void*> blocks;
   size_t bytes = 0;
+  bool failed = false;   // a request was refused: whoever made it stops before its next launch
   void* get(size_t n);
   void release_all();
 };

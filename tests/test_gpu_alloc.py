@@ -1,0 +1,69 @@
+"""Creating a handle on an allocator that runs out: the create reports it, or
+goes without the buffers that a solve can do without."""
+import pytest
+
+from paper_2606_17636_gb300 import workloads
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ps():
+    import paper_2606_17636_gb300 as m
+    m.lib()
+    return m
+
+
+def _create(ps, monkeypatch, refuse, spec, **kw):
+    """A solver (or None when the create fails for want of memory) whose
+    allocator refuses where refuse(index of the request, bytes, bytes held)."""
+    class Allocator(ps._TorchAllocator):
+        def __init__(self):
+            super().__init__()
+            self.sizes, self.peak = [], 0
+
+        def _alloc(self, nbytes, user):
+            held = sum(t.numel() for t in self.live.values())
+            self.sizes.append(nbytes)
+            if refuse(len(self.sizes) - 1, nbytes, held):
+                return None
+            self.peak = max(self.peak, held + nbytes)
+            return super()._alloc(nbytes, user)
+
+    monkeypatch.setattr(ps, "_TorchAllocator", Allocator)
+    try:
+        return ps.Solver.from_spec(spec, **kw)
+    except ps.PSolveError as e:
+        assert e.code == ps.ERR_NOMEM
+        return None
+
+
+SPECS = {
+    # levels above the shared-memory ones, auxiliary windows
+    "wide": (dict(precision=1), workloads.spec(workloads.CYLINDRICAL, 256, 32, 4, workloads.UNIFORM, 1.0, 3.0, 0.0, 0.25)),
+    "fp64": (dict(precision=0), workloads.spec(workloads.SPHERICAL, 32, 32, 4, workloads.UNIFORM, 1.0, 2.0)),
+    # the extended-domain tables, whose set-up solves on planes of its own
+    "extended": (dict(precision=1), workloads.spec(workloads.SPHERICAL, 32, 32, 4, workloads.LOG, 0.1, 10.0)),
+}
+
+
+@pytest.mark.parametrize("key", list(SPECS))
+def test_a_refused_request_is_reported_or_done_without(ps, monkeypatch, key):
+    """Each request in turn is refused and the later ones granted: no kernel may
+    run on a missing buffer."""
+    kw, sp = SPECS[key]
+    rho = torch.rand((sp["n_r"], sp["n_tz"], sp["n_phi"]), dtype=torch.float64, device="cuda")
+    s = _create(ps, monkeypatch, lambda k, n, held: False, sp, **kw)
+    ref = s.solve(rho, tol=1e-9)[0].clone()
+    requests = len(s._alloc.sizes)
+    s.close()
+    without = 0
+    for q in range(requests):
+        s = _create(ps, monkeypatch, lambda k, n, held: k == q, sp, **kw)
+        torch.cuda.synchronize()
+        if s is not None:
+            without += 1
+            assert torch.equal(s.solve(rho, tol=1e-9)[0], ref)
+            s.close()
+    assert without < requests // 4
