@@ -51,7 +51,16 @@ enum {
  * from alloc(bytes, user) and returned with free(ptr, user); otherwise
  * cudaMalloc / cudaFree are used.  alloc returns NULL on failure, and
  * 256-byte aligned memory otherwise (as cudaMalloc does); a block that is not
- * so aligned is handed back to free and counts as a failed allocation. */
+ * so aligned is handed back to free and counts as a failed allocation.
+ * Besides the boundary tables (8 bytes per mode and pair of boundary points) a
+ * handle needs about 70 bytes per cell, mode and density (PSOLVE_MIXED) or 100
+ * (PSOLVE_FP64).  After everything that it needs it asks for what only makes
+ * solves faster, with the same bits: a second set of error planes of the levels
+ * above the fused ones (PSOLVE_MIXED, 8 to 11 bytes per cell, mode and density),
+ * the inverse diagonals of the smoothed levels (PSOLVE_FP64, up to 22 bytes per
+ * cell and mode).  A refusal there costs speed alone.  alloc decides by itself;
+ * from cudaMalloc they are taken where they need at most an eighth of the device
+ * memory that is free. */
 typedef void* (*psolve_alloc_fn)(size_t bytes, void* user);
 typedef void (*psolve_free_fn)(void* ptr, void* user);
 

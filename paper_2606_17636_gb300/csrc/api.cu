@@ -310,6 +310,10 @@ static int create_impl(psolve_t* out, const psolve_desc* din, int nd) {
                   "DGF: " + err);
     }
   }
+  if (!h->mg.optional_buffers(h->A, err)) {
+    h->A.release_all();
+    return fail(PSOLVE_ERR_CUDA, "create: " + err);
+  }
   if (!cuda_ok("create")) {
     h->A.release_all();
     return PSOLVE_ERR_CUDA;

@@ -143,6 +143,7 @@ static bool build_extended(const PlaneGeo& g, const Law& rlaw, const Law& tlaw,
   double2* u = static_cast<double2*>(A.get(sizeof(double2) * cells * chunk));
   double2* f = static_cast<double2*>(A.get(sizeof(double2) * cells * chunk));
   if (A.failed) { err = "out of device memory (DGF planes)"; return false; }
+  if (!mg.optional_buffers(A, err)) return false;
   for (long p0 = 0; p0 < total; p0 += chunk) {
     const int np = int(std::min<long>(chunk, total - p0));
     for (int p = 0; p < np; ++p) slot[p] = int((p0 + p) / ea.npairs);

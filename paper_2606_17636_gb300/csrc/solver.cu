@@ -11,7 +11,7 @@
 
 namespace ps {
 
-void* Arena::get(size_t n) {
+void* Arena::get(size_t n, bool optional) {
   if (n == 0) n = 16;
   n = (n + 255) & ~size_t(255);
   void* p = nullptr;
@@ -27,10 +27,18 @@ void* Arena::get(size_t n) {
   if (p) {
     blocks.push_back(p);
     bytes += n;
-  } else {
+  } else if (!optional) {
     failed = true;
   }
   return p;
+}
+
+void Arena::give_back(void* p) {
+  const auto at = std::find(blocks.begin(), blocks.end(), p);
+  if (!p || at == blocks.end()) return;
+  blocks.erase(at);
+  if (free_fn) free_fn(p, user);
+  else cudaFree(p);
 }
 
 void Arena::release_all() {
@@ -220,6 +228,56 @@ bool MGSolver::build_vsmem(Arena& A, int lo, int n_modes, VSmemArgs& v, std::str
   return true;
 }
 
+// Buffers that make a solve faster and that it can do without, with bitwise the
+// same result.  Asked for when everything that a handle needs is there: requested
+// before the last of that, they made a create fail that fits without them.
+//  - FP64: inverse diagonals per mode and cell of the levels on the line passes
+//    (which form them otherwise).
+//  - Mixed: the window passes' second set of error buffers (without them every
+//    plane stays with the level-wide passes).
+// An allocator of the caller's decides by itself whether it grants them; from
+// cudaMalloc they are taken where they need at most an eighth of the free memory.
+bool MGSolver::optional_buffers(Arena& A, std::string& err) {
+  size_t need = 0, free_b = 0, total_b = 0;
+  const size_t S_ = H.lv[0].om_r.size() / size_t(lv[0].nt);   // mode slots
+  auto cells = [&](int l) { return size_t(lv[l].nr) * lv[l].nt; };
+  for (int l = 0; l < base; ++l) need += opt.precision ? size_t(max_planes) * cells(l) * vbytes() : 2 * sizeof(double) * S_ * cells(l);
+  if (!need) return true;
+  if (!A.alloc_fn && (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || need > free_b / 8)) {
+    cudaGetLastError();
+    return true;
+  }
+  if (opt.precision) {
+    std::vector<void*> x(base, nullptr);
+    for (int l = 0; l < base; ++l)
+      if (!(x[l] = A.get(size_t(max_planes) * cells(l) * vbytes(), true))) {
+        while (l-- > 0) A.give_back(x[l]);
+        cudaGetLastError();
+        return true;
+      }
+    tmp2 = x[0];
+    e2.assign(H.lv.size(), nullptr);
+    for (int l = 1; l < base; ++l) e2[l] = x[l];
+    plan_tiles();
+    return true;
+  }
+  for (int l = 0; l < base; ++l) {
+    double* a = static_cast<double*>(A.get(sizeof(double) * S_ * cells(l), true));
+    double* b = static_cast<double*>(A.get(sizeof(double) * S_ * cells(l), true));
+    if (!a || !b) {
+      A.give_back(a);
+      A.give_back(b);
+      break;
+    }
+    launch_inverse_diagonal(lv[l], d_s2, int(S_), a, b, 0);
+    lv[l].idr = a;
+    lv[l].idt = b;
+  }
+  cudaGetLastError();
+  if (cudaStreamSynchronize(0) != cudaSuccess) { err = "inverse diagonals"; return false; }
+  return true;
+}
+
 bool MGSolver::init(Arena& A, const PlaneGeo& fine, bool neumann, const std::vector<int>& modes,
                     const std::vector<int>& plane_slot, int mp, const MGOptions& o,
                     std::string& err) {
@@ -335,43 +393,6 @@ bool MGSolver::init(Arena& A, const PlaneGeo& fine, bool neumann, const std::vec
     // keeps the levels together: its passes are short of FP32 work, not SMs.
     base = nl - 1;
     if (!build_vsmem(A, base, int(modes.size()), vsb, err)) return false;
-  }
-  if (A.failed) { err = "out of device memory"; return false; }
-  if (!opt.precision) {
-    // FP64 smoothing: inverse diagonals per mode and cell of the levels on the
-    // line passes, where they take at most an eighth of the free memory (the
-    // passes form them otherwise)
-    size_t need = 0, free_b = 0, total_b = 0;
-    for (int l = 0; l < base; ++l) need += 2 * sizeof(double) * modes.size() * size_t(lv[l].nr) * lv[l].nt;
-    if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && need <= free_b / 8) {
-      for (int l = 0; l < base; ++l) {
-        const size_t bytes = sizeof(double) * modes.size() * size_t(lv[l].nr) * lv[l].nt;
-        double* a = static_cast<double*>(A.get(bytes));
-        double* b = static_cast<double*>(A.get(bytes));
-        if (!a || !b) {   // the passes do without
-          A.failed = false;
-          break;
-        }
-        launch_inverse_diagonal(lv[l], d_s2, int(modes.size()), a, b, 0);
-        lv[l].idr = a;
-        lv[l].idt = b;
-      }
-      cudaGetLastError();
-      if (cudaStreamSynchronize(0) != cudaSuccess) { err = "inverse diagonals"; return false; }
-    }
-  }
-  if (opt.precision && base > 0) {   // the window passes' buffers; without them every plane stays with the level-wide passes
-    tmp2 = A.get(size_t(mp) * lv[0].nr * lv[0].nt * vb);
-    e2.assign(nl, nullptr);
-    for (int l = 1; l < base && tmp2; ++l) {
-      e2[l] = A.get(size_t(mp) * lv[l].nr * lv[l].nt * vb);
-      if (!e2[l]) tmp2 = nullptr;
-    }
-    if (!tmp2) {
-      A.failed = false;
-      cudaGetLastError();
-    }
-    plan_tiles();
   }
   const int nblk = residual_blocks(lv[0].nr, lv[0].nt);
   d_act = static_cast<int*>(A.get(sizeof(int) * mp));

@@ -14,8 +14,9 @@ struct Arena {
   void* user = nullptr;
   std::vector<void*> blocks;
   size_t bytes = 0;
-  bool failed = false;   // a request was refused: whoever made it stops before its next launch
-  void* get(size_t n);
+  bool failed = false;   // a needed request was refused: whoever made it stops before its next launch
+  void* get(size_t n, bool optional = false);
+  void give_back(void* p);
   void release_all();
 };
 
@@ -49,6 +50,8 @@ class MGSolver {
   bool init(Arena& A, const PlaneGeo& fine, bool neumann, const std::vector<int>& modes,
             const std::vector<int>& plane_slot, int max_planes, const MGOptions& o,
             std::string& err);
+  // What a solve can do without, asked for last (false: a CUDA call failed).
+  bool optional_buffers(Arena& A, std::string& err);
   // Solve L u = f for all planes (u holds the initial guess).  Enqueued on
   // st; with cond_handle (use_cond) the loop is a graph WHILE body; in eager
   // mode the host reads the continue flag each iteration.

@@ -12,13 +12,14 @@ pytestmark = pytest.mark.gpu
 def ps():
     import paper_2606_17636_gb300 as m
     m.lib()
+    _create.base = m._TorchAllocator
     return m
 
 
 def _create(ps, monkeypatch, refuse, spec, **kw):
     """A solver (or None when the create fails for want of memory) whose
     allocator refuses where refuse(index of the request, bytes, bytes held)."""
-    class Allocator(ps._TorchAllocator):
+    class Allocator(_create.base):
         def __init__(self):
             super().__init__()
             self.sizes, self.peak = [], 0
@@ -67,3 +68,29 @@ def test_a_refused_request_is_reported_or_done_without(ps, monkeypatch, key):
             assert torch.equal(s.solve(rho, tol=1e-9)[0], ref)
             s.close()
     assert without < requests // 4
+
+
+@pytest.mark.parametrize("key,optional", [("wide", 1), ("fp64", 2)])
+def test_a_create_that_fits_without_the_optional_buffers(ps, monkeypatch, key, optional):
+    """The window passes' buffer (mixed) and the stored inverse diagonals (FP64)
+    are asked for last: an allocator with room for everything else, and no more,
+    gives a working handle with the same result."""
+    kw, sp = SPECS[key]
+    rho = torch.rand((sp["n_r"], sp["n_tz"], sp["n_phi"]), dtype=torch.float64, device="cuda")
+    s = _create(ps, monkeypatch, lambda k, n, held: False, sp, **kw)
+    requests = len(s._alloc.sizes)
+    ref = s.solve(rho, tol=1e-9)[0].clone()
+    if key == "wide":
+        assert s.loops()["few_planes"] > 0
+    s.close()
+    s = _create(ps, monkeypatch, lambda k, n, held: k >= requests - optional, sp, **kw)
+    assert s is not None and len(s._alloc.sizes) in range(requests - optional + 1, requests + 1)
+    room = s._alloc.peak
+    if key == "wide":
+        assert s.loops()["few_planes"] == 0
+    assert torch.equal(s.solve(rho, tol=1e-9)[0], ref)
+    s.close()
+    s = _create(ps, monkeypatch, lambda k, n, held: held + n > room, sp, **kw)
+    assert s is not None
+    assert torch.equal(s.solve(rho, tol=1e-9)[0], ref)
+    s.close()
