@@ -48,7 +48,7 @@ static int grid_rows(int base, int planes) {
 // pass: 32.8 / 33.9 us, 40.7 / 40.8 with the diagonal formed in the pass; one
 // plane 9.8 / 7.2, 11.8 / 8.0.
 template <typename T, int CPL>
-constexpr bool kIds = sizeof(T) == 8 && CPL <= 8;
+constexpr bool kIds = sizeof(T) == 8 && reads_inverse_diagonal(32 * CPL);
 
 // Radial pass, both colours: a block of 32 Wmax threads owns W lines
 // [j0, j0+W), W = Wmax / mult.
@@ -374,8 +374,8 @@ __global__ void k_inverse_diagonal(LevelDev L, const double* __restrict__ s2d, i
     const double d = fmac(-(s2d[slot] * L.rd[RT_Q * NR + i + 1]), L.td[TT_T * NT + j + 1],
                           fmac(L.rd[RT_P * NR + i + 1], L.td[TT_DT * NT + j + 1], L.rd[RT_DR * NR + i + 1]));
     const double v = rcp_diag(d);   // the passes' own value
-    idr[q] = v;
-    idt[(slot * nr + i) * nt + j] = v;
+    if (idr) idr[q] = v;
+    if (idt) idt[(slot * nr + i) * nt + j] = v;
   }
 }
 

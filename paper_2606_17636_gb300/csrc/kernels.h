@@ -192,7 +192,9 @@ struct LevelDev {
   const double* idr = nullptr;
   const double* idt = nullptr;
 };
-// Fills them (device pointers) from the level's tables.
+// Whether the passes along lines of n cells read them.
+constexpr bool reads_inverse_diagonal(int n) { return n <= 256; }
+// Fills them (device pointers, null: not that one) from the level's tables.
 void launch_inverse_diagonal(const LevelDev& L, const double* s2d, int slots, double* idr, double* idt, cudaStream_t st);
 
 // A batch of planes: plane p of a level buffer starts at p * nr * nt; its

@@ -241,7 +241,9 @@ bool MGSolver::optional_buffers(Arena& A, std::string& err) {
   size_t need = 0, free_b = 0, total_b = 0;
   const size_t S_ = H.lv[0].om_r.size() / size_t(lv[0].nt);   // mode slots
   auto cells = [&](int l) { return size_t(lv[l].nr) * lv[l].nt; };
-  for (int l = 0; l < base; ++l) need += opt.precision ? size_t(max_planes) * cells(l) * vbytes() : 2 * sizeof(double) * S_ * cells(l);
+  for (int l = 0; l < base; ++l)
+    need += opt.precision ? size_t(max_planes) * cells(l) * vbytes()
+                          : sizeof(double) * S_ * cells(l) * (reads_inverse_diagonal(lv[l].nr) + reads_inverse_diagonal(lv[l].nt));
   if (!need) return true;
   if (!A.alloc_fn && (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || need > free_b / 8)) {
     cudaGetLastError();
@@ -262,14 +264,16 @@ bool MGSolver::optional_buffers(Arena& A, std::string& err) {
     return true;
   }
   for (int l = 0; l < base; ++l) {
-    double* a = static_cast<double*>(A.get(sizeof(double) * S_ * cells(l), true));
-    double* b = static_cast<double*>(A.get(sizeof(double) * S_ * cells(l), true));
-    if (!a || !b) {
+    const size_t bytes = sizeof(double) * S_ * cells(l);
+    const bool want_r = reads_inverse_diagonal(lv[l].nr), want_t = reads_inverse_diagonal(lv[l].nt);
+    double* a = want_r ? static_cast<double*>(A.get(bytes, true)) : nullptr;
+    double* b = want_t ? static_cast<double*>(A.get(bytes, true)) : nullptr;
+    if ((want_r && !a) || (want_t && !b)) {
       A.give_back(a);
       A.give_back(b);
       break;
     }
-    launch_inverse_diagonal(lv[l], d_s2, int(S_), a, b, 0);
+    if (a || b) launch_inverse_diagonal(lv[l], d_s2, int(S_), a, b, 0);
     lv[l].idr = a;
     lv[l].idt = b;
   }

@@ -94,3 +94,16 @@ def test_a_create_that_fits_without_the_optional_buffers(ps, monkeypatch, key, o
     assert s is not None
     assert torch.equal(s.solve(rho, tol=1e-9)[0], ref)
     s.close()
+
+
+@pytest.mark.parametrize("nr,nt,arrays", [(64, 32, 2), (512, 32, 1), (32, 512, 1)])
+def test_fp64_diagonals_only_where_lines_read_them(ps, monkeypatch, nr, nt, arrays):
+    """The FP64 passes read stored inverse diagonals along lines of up to 256
+    cells: the finest level asks for one array per such direction (besides the
+    residual's diagonal of the same size)."""
+    sp = workloads.spec(workloads.CYLINDRICAL, nr, nt, 8, workloads.UNIFORM, 1.0, 3.0, 0.0, 2.0 * nt / nr)
+    s = _create(ps, monkeypatch, lambda k, n, held: False, sp, precision=0)
+    want = 8 * s.n_modes * nr * nt
+    tail = s._alloc.sizes[-12:]
+    assert tail.count(want) == arrays
+    s.close()
