@@ -347,8 +347,10 @@ int psolve_set_schedule(psolve_t h, const psolve_schedule* s);
  * timed solves (CUDA events on the handle's stream); its time is their
  * median.  Candidates whose solve fails are skipped, and so are those whose
  * potential is further (relative 2-norm) from a solve to tol / 1000 with the
- * handle's current schedule than 10 tol and than that schedule's own at tol (no
- * limit when that residual cannot be reached or its copy does not fit).  Warm start is
+ * handle's current schedule (its last iterate where that residual is out of reach)
+ * than 10 tol and than that schedule's own at tol.  When that solve gives no finite
+ * potential the current schedule stays; when its copy does not fit there is no
+ * limit.  Warm start is
  * suspended while tuning (the history is kept).  phi (device, caller-owned)
  * receives the last solve's potential.
  * Choices are cached per process by the key (geometry, sizes, spacing,

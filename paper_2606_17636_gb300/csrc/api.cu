@@ -1091,15 +1091,17 @@ __global__ void __launch_bounds__(256) k_distance(const double* __restrict__ a, 
   }
 }
 
-// A candidate's potential against a much tighter solve of the same density: a
-// schedule that leaves a smooth final residual meets the residual tolerance
-// with a larger error (256 x 64 x 8, tolerance 1e-8: relative errors from
-// 2e-8 to 2.5e-7), so speed alone does not choose.
+// A candidate's potential against a tighter solve of the same density: a schedule
+// that leaves a smooth final residual meets the residual tolerance with a larger
+// error (256 x 64 x 8, tolerance 1e-8: relative errors from 2e-8 to 2.5e-7), so
+// speed alone does not choose.  Where that residual is out of reach, the last
+// iterate of the attempt is still the nearest potential there is.
 struct TuneGuard {
   psolve_t h;
   Arena mem;
   double *ref = nullptr, *sums = nullptr;
-  double limit = INFINITY;
+  bool have = false;    // ref holds a potential
+  double limit = -1.0;  // set by the handle's own schedule; none passes before
   size_t n;
   TuneGuard(psolve_t h_, const double* rho, double* phi, double tol) : h(h_), n(size_t(h_->nd) * cells(h_)) {
     mem.alloc_fn = h->A.alloc_fn;
@@ -1113,26 +1115,27 @@ struct TuneGuard {
     sums = ref + n;
     int rc = enqueue_solve(h, rho, phi, 1e-3 * tol);
     if (rc == PSOLVE_OK) rc = finish(h);
-    if (rc != PSOLVE_OK || cudaMemcpyAsync(ref, phi, n * sizeof(double), cudaMemcpyDeviceToDevice, h->st) != cudaSuccess) {
-      mem.release_all();   // beyond the reachable residual
-      ref = nullptr;
-    }
+    if (rc == PSOLVE_OK || rc == PSOLVE_ERR_NOT_CONVERGED)
+      have = cudaMemcpyAsync(ref, phi, n * sizeof(double), cudaMemcpyDeviceToDevice, h->st) == cudaSuccess;
   }
   ~TuneGuard() { mem.release_all(); }
+  // relative 2-norm; not a number when it could not be had
   double distance(const double* phi) const {
-    if (!ref) return 0.0;
-    double v[2] = {0.0, 0.0};
+    double v[2] = {NAN, NAN};
     cudaMemsetAsync(sums, 0, 2 * sizeof(double), h->st);
     k_distance<<<unsigned(std::min<size_t>((n + 255) / 256, 1024)), 256, 0, h->st>>>(phi, ref, n, sums);
-    cudaMemcpyAsync(v, sums, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->st);
-    if (cudaStreamSynchronize(h->st) != cudaSuccess) return 0.0;
-    return v[1] > 0.0 ? std::sqrt(v[0] / v[1]) : 0.0;
+    if (cudaMemcpyAsync(v, sums, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->st) != cudaSuccess ||
+        cudaStreamSynchronize(h->st) != cudaSuccess)
+      return NAN;
+    return v[0] == 0.0 ? 0.0 : std::sqrt(v[0] / v[1]);
   }
   // the first solve (the handle's own schedule) sets the limit
   bool accept(const double* phi, double tol, bool first) {
+    if (!ref) return true;
+    if (!have) return false;
     const double d = distance(phi);
-    if (first) limit = std::fmax(d, 10.0 * tol);
-    return !(d > limit);
+    if (first && std::isfinite(d)) limit = std::fmax(d, 10.0 * tol);
+    return d <= limit;
   }
 };
 

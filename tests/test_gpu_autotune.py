@@ -170,3 +170,27 @@ def test_autotune_reports_a_failing_solve_and_keeps_the_schedule(ps):
     assert e.value.code == ps.ERR_NOT_CONVERGED
     assert s.schedule() == before
     s.close()
+
+
+@pytest.mark.parametrize("tol,r_out", [(1e-10, 10.04), (1e-11, 10.05)])
+def test_autotune_holds_the_answer_where_a_much_tighter_solve_is_out_of_reach(ps, tol, r_out):
+    """At tolerances whose thousandth part the residual cannot reach, the choice
+    still gives an error of at most ten times the tolerance or of the handle's own
+    schedule (here an accurate one), both against the last iterate of an FP64 solve
+    beyond its reachable residual; half a tolerance on top for that reference and
+    the tuner's own."""
+    from paper_2606_17636_gb300 import workloads as wl
+    sp = _spec(wl.SPHERICAL, 256, 64, 8, wl.LOG, 0.1, r_out)
+    rho = torch.from_numpy(clumps(sp, 43)).cuda()
+    ref64 = ps.Solver.from_spec(sp, precision=ps.FP64)
+    tight = ref64.solve(rho, tol=1e-14, raise_on_error=False)[0].clone()
+    ref64.close()
+    s = ps.Solver.from_spec(sp, precision=ps.MIXED)
+    s.set_schedule(3, 3, 3)
+    assert s.solve(rho, tol=1e-3 * tol, raise_on_error=False)[1] == ps.ERR_NOT_CONVERGED
+    own = _rel(s.solve(rho, tol=tol)[0], tight)
+    ch = s.autotune(rho, tol=tol)
+    assert ch["cached"] == 0
+    err = _rel(s.solve(rho, tol=tol)[0], tight)
+    assert err <= max(own, 10 * tol) + 0.5 * tol, (err, own, ch)
+    s.close()
