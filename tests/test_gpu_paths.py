@@ -219,3 +219,34 @@ def test_fp64_solves_with_stored_inverse_diagonals(ps, nr, nt, n_phi):
         assert np.abs(u[m].cpu().numpy() - ref).max() <= 1e-10 * np.abs(ref).max()
         assert abs(cyc[m] - H.solve(m, b, 1e-12)[1]) <= 1
     s.close()
+
+
+# finest level, schedule, whether the halo of one smoothing cycle (4 n_sor + 1 cells,
+# one more for the restriction) leaves a 64-cell window 16 cells of its own
+WINDOWS = [(256, 128, (2, 1, 2, 3, 1), True), (256, 128, (2, 2, 3, 0, 0), True), (256, 128, (2, 2, 5, 0, 0), True),
+           (512, 256, (2, 2, 2, 0, 0), True), (512, 32, (2, 2, 2, 0, 0), True), (256, 128, (2, 2, 6, 0, 0), False)]
+
+
+@pytest.mark.parametrize("nr,nt,sched,windows", WINDOWS)
+def test_window_passes_run_where_they_fit_also_in_a_captured_solve(ps, nr, nt, sched, windows):
+    """The handle says whether a solve's last planes take the window passes, and a
+    captured solve (two loops with a hand-over, several iterations per pass) gives
+    the bits and cycle counts of the eager one."""
+    from gpu_helpers import clumps
+    sp = workloads.spec(workloads.CYLINDRICAL, nr, nt, 64, workloads.UNIFORM, 1.0, 3.0, 0.0, 2.0 * nt / nr)
+    rho = torch.from_numpy(clumps(sp, 3)).cuda()
+    out = []
+    for graph in (False, True):
+        s = ps.Solver.from_spec(sp, precision=ps.MIXED, use_graph=graph)
+        s.set_schedule(*sched[:3], nu_pre_fused=sched[3], nu_post_fused=sched[4])
+        few = s.loops()["few_planes"]
+        assert (few > 0) == windows
+        # 33 planes hand over from the level-wide passes, but for 512 x 32 cells, whose planes all fit
+        assert few < s.n_modes or (nr, nt) == (512, 32)
+        phi, rc = s.solve(rho, tol=1e-8)
+        assert rc == ps.OK
+        st = s.stats()
+        out.append((phi.clone(), st["cycles_psi"], st["cycles_phi"]))
+        assert sum(1 for c in st["cycles_phi"] if c == max(st["cycles_phi"])) < s.n_modes
+        s.close()
+    assert torch.equal(out[0][0], out[1][0]) and out[0][1:] == out[1][1:]
