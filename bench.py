@@ -651,17 +651,17 @@ def launches_per_solve(s, st):
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of full-batch
 # launches on workload 3 (all 129 modes), from the ncu captures of the
 # profiling case (python -m paper_2606_17636_gb300.profile_case
-# --schedule 2,1,2,4,16,2,2 --smooth-first): one k_vpatch launch, one
+# --smooth-first): one k_vpatch launch, one
 # finest-level smoothing cycle (k_band + k_march) and the first stencil
 # launch of k_residual.  They hold for the kernels as captured; a changed
 # kernel needs a new capture.
-VSMEM_TRAFFIC_BYTES = 13771520
-SMOOTH_CYCLE_TRAFFIC_BYTES = 67737344 + 2694656 + 69978624 + 5459712
-RESIDUAL_TRAFFIC_BYTES = 169805568 + 23041280
+VSMEM_TRAFFIC_BYTES = 13771776
+SMOOTH_CYCLE_TRAFFIC_BYTES = 67737344 + 3030016 + 70557184 + 5885440
+RESIDUAL_TRAFFIC_BYTES = 169818880 + 21721344
 # ncu sm__inst_executed_pipe_fp64 (percent of peak, sustained active) of the
 # kernels bound by the FP64 pipe: k_residual from the same capture at 256 x
 # 128 x 256, k_boundary at 256 x 128 x 128 (the same kernel, 65 mode planes)
-FP64_PIPE_PCT = {"k_residual": 77.6, "k_boundary": 87.1}
+FP64_PIPE_PCT = {"k_residual": 79.3, "k_boundary": 87.1}
 
 
 def vcycle_flops_per_cell(sched):

@@ -448,11 +448,14 @@ int psolve_stage_residual(psolve_t h, int precision, const double* f, const doub
  * psolve_get_fused_level) down to the coarsest, on L_m e = f with a zero
  * initial guess: nu_pre smoothing cycles, defect restriction, recursion,
  * the direct coarsest solve (see psolve_desc.coarsest_size), prolongation,
- * nu_post smoothing cycles.
+ * nu_post smoothing cycles.  A PSOLVE_MIXED solve runs this kernel; a PSOLVE_FP64
+ * solve smooths these levels with the level-wide passes and leaves it the coarsest
+ * solve alone (psolve_loops.level_wide), so in FP64 its time is not a solve's.
  * f, e: planes [M][n_tz_l][n_r_l] complex in FP64 (precision 0) or FP32 (1);
  * e is overwritten.  PSOLVE_ERR_ARG for another level or precision. */
 int psolve_stage_vcycle(psolve_t h, int level, int precision, const void* f, void* e);
-/* The first multigrid level held in shared memory by the fused V-cycle. */
+/* The first multigrid level that the fused V-cycle can hold on chip: where
+ * psolve_stage_vcycle starts. */
 int psolve_get_fused_level(psolve_t h, int* level);
 /* Eqs. charge_sph / charge_cyl: sigma[m][b] (complex) from psi_hat. */
 int psolve_stage_screening(psolve_t h, const double* psi_hat, double* sigma);

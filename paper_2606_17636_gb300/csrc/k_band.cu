@@ -398,7 +398,11 @@ void march(const LevelDev& L, const Batch& B, const float2* ein, float2* eout, c
 // 1.5 M cells over all planes the staged passes' shorter way through a launch
 // wins by 1 to 2 us a pass (64 x 64 x 33 planes, two cycles: 43 us against 44;
 // 128 x 64 x 129: 62 against 67; above, 256 x 64 x 129: 88 against 79,
-// 256 x 128 x 129: 168 against 116, 512 x 256 x 33: 206 against 150).
+// 256 x 128 x 129: 168 against 116, 512 x 256 x 33: 206 against 150).  planes
+// counts the batch, not the active ones: above the line the register passes also
+// win with few planes active (an iteration's smoothing and update, staged against
+// here: 17 of 129 planes of 256 x 128 92 and 65 us, 6 of 65 of 512 x 256 200 and
+// 145, 33 of 257 of 256 x 64 84 and 64).
 bool band_pays(int nr, int nt, int n_sor, int planes) {
   return run_length(nr) && run_length(nt) && n_sor >= 1 && n_sor <= 3 && long(planes) * nr * nt >= 1500000l;
 }

@@ -10,10 +10,11 @@
 // for 256 x 128 rows of 256 values (152 us of pipe time at best for
 // 5 N log2 N operations), where the bytes take 20 us.  In fixed point an
 // addition is two integer instructions and a twiddle product twelve 32-bit
-// multiplies; the same transforms take 61 and 79 us, bound by the issue of warp
-// instructions (16 warps an SM at 128 registers).  Zero times a twiddle is zero, so
-// that modes which cancel exactly, those of rows constant or periodic along phi,
-// come out as zeros and retire at their first residual.
+// multiplies; the same transforms take 61 and 79 us, bound by the issue of 41 and
+// 54 million warp instructions (integer ALU pipe 56 % busy, 16 warps an SM at 128
+// registers).  Zero times a twiddle is zero, so that modes which cancel exactly,
+// those of rows constant or periodic along phi, come out as zeros and retire at
+// their first residual.
 //
 // Scaling: a row's values are aligned to its largest exponent (a power of two
 // each, so scaling a row scales its spectrum exactly).  Every partial sum of a

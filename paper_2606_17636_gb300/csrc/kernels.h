@@ -76,9 +76,9 @@ __device__ __forceinline__ double f32_to_f64(float x) {
 }
 // The same for streams of values (the refinement's update): the cases beyond
 // normal values and zero behind a call, so that the common ones take six
-// instructions instead of the 20 and more of all cases as selects.  Update
-// fused into the polar march, 129 planes of 256 x 128: 66 -> 61 us, one
-// plane 10.0 -> 8.7.  (Kernels that are short of registers keep the form above.)
+// instructions instead of the 20 and more of all cases as selects (8 % of a
+// polar pass over 129 planes of 256 x 128 cells that also updated, a launch that
+// is now two).  Kernels that are short of registers keep the form above.
 static __device__ __noinline__ double f32_to_f64_rare(float x) { return f32_to_f64(x); }
 __device__ __forceinline__ double widen(float x) {
   const unsigned b = __float_as_uint(x), a = b & 0x7fffffffu;
